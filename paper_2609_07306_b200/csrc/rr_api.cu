@@ -81,20 +81,19 @@ RRParams shape_params(const rr_config* cfg) {
   return p;
 }
 
-// The two-sweep kernel wins where the grid fills the GPU several times over (its per-score work
-// is smaller); on grids of less than two waves of CTAs a layer is a chain of kernel latencies,
-// and the streaming kernel -- one sweep, sentinels inside, one launch less -- is the shorter
-// chain (measured on the 32-problem chunk sweep: 5-10 % per step).  148 SMs, one CTA per SM.
+// Which kernel routes rows.  Two threads per row with two CTAs per SM (rr_route_rows.cu) wherever
+// its shape limits hold; the relay in place (debug bit 5) exists in the four-threads-per-row kernel
+// only; the streaming kernel takes wider routes (and debug bit 4), the two-pass path the rest.
 bool uses_sweep(const rr_config* cfg) {
-  if (cfg->debug_outputs & (2 | 16)) return false;
-  const RRParams p = shape_params(cfg);
-  if (!rr_route_sweep_supported(p)) return false;
-  const bool forced = (cfg->debug_outputs & (32 | 256)) != 0;   // relay in place needs it; bit 8 asks for it
-  return forced || p.n_tiles >= 2 * 148 || !rr_route_fused_supported(p);
+  return (cfg->debug_outputs & 32) && !(cfg->debug_outputs & (2 | 16)) && rr_route_sweep_supported(shape_params(cfg));
+}
+
+bool uses_rows(const rr_config* cfg) {
+  return !(cfg->debug_outputs & (2 | 16)) && !uses_sweep(cfg) && rr_route_rows_supported(shape_params(cfg));
 }
 
 bool uses_fused(const rr_config* cfg) {
-  return !(cfg->debug_outputs & 2) && !uses_sweep(cfg) && rr_route_fused_supported(shape_params(cfg));
+  return !(cfg->debug_outputs & 2) && !uses_sweep(cfg) && !uses_rows(cfg) && rr_route_fused_supported(shape_params(cfg));
 }
 
 Layout make_layout(const rr_config* c) {
@@ -126,7 +125,7 @@ Layout make_layout(const rr_config* c) {
   L.token_ranges = o;    o = align_up(o + (c->chunk_tokens > 0 ? rows * c->k * 8 : 0));
   L.cand_scores = o;     o = align_up(o + ((c->debug_outputs & 1) ? rows * cw * 4 : 0));
   // score rows are only materialised by the two-pass path
-  L.S = o;               o = align_up(o + (uses_fused(c) || uses_sweep(c) ? 0 : rows * (size_t)c->n_k * 4));
+  L.S = o;               o = align_up(o + (uses_fused(c) || uses_sweep(c) || uses_rows(c) ? 0 : rows * (size_t)c->n_k * 4));
   L.scratch_total = o;
   return L;
 }
@@ -169,7 +168,9 @@ int route_layer(rr_ledger* L, const void* qc, const void* kc, int layer, bool an
   if (anchor) {
     // Section 4.1: the anchor builds the state from a complete chunk-score matrix.
     LAUNCH(RR_KIND_ANCHOR_FILL, rr_launch_anchor_fill(p, L->dense_pairs_per_layer, st));
-    if (L->sweep) {
+    if (L->rows) {
+      LAUNCH(RR_KIND_ROUTE_FUSED, rr_launch_route_rows(p, qc, kc, nullptr, layer, sweep_hooks(L), st));
+    } else if (L->sweep) {
       LAUNCH(RR_KIND_ROUTE_FUSED, rr_launch_route_sweep(p, qc, kc, nullptr, layer, 0,
                                                         sweep_hooks(L), st));
       LAUNCH(RR_KIND_SENTINELS, rr_launch_sentinels(p, nullptr, layer, st));
@@ -198,11 +199,13 @@ int route_layer(rr_ledger* L, const void* qc, const void* kc, int layer, bool an
     if (L->dense_rescore) {
       const int shot = (L->timeout_shots >> 1) & 1;     // test hook: one forced time-out
       L->timeout_shots &= ~2;
-      LAUNCH(RR_KIND_RESCORE_DENSE, rr_launch_rescore_dense(p, qc, kc, shot, /*prior=*/!L->sweep, st));
+      LAUNCH(RR_KIND_RESCORE_DENSE, rr_launch_rescore_dense(p, qc, kc, shot, /*prior=*/L->fused, st));
     }
     else LAUNCH(RR_KIND_RESCORE, rr_launch_rescore(p, qc, kc, st));
     LAUNCH(RR_KIND_COMPACT, rr_launch_compact(p, L->dense_pairs_per_layer, st));
-    if (L->sweep) {
+    if (L->rows) {
+      LAUNCH(RR_KIND_ROUTE_FUSED, rr_launch_route_rows(p, qc, kc, p.refresh_rows, layer, sweep_hooks(L), st));
+    } else if (L->sweep) {
       LAUNCH(RR_KIND_ROUTE_FUSED, rr_launch_route_sweep(p, qc, kc, p.refresh_rows, layer, 0,
                                                         sweep_hooks(L), st));
       LAUNCH(RR_KIND_SENTINELS, rr_launch_sentinels(p, p.refresh_rows, layer, st));
@@ -291,6 +294,7 @@ int rr_ledger_init(const rr_config* cfg, void* dev_ledger, size_t ledger_bytes,
   p.token_ranges = cfg->chunk_tokens > 0 ? (int32_t*)(sb + lay.token_ranges) : nullptr;
   p.cand_scores = (cfg->debug_outputs & 1) ? (float*)(sb + lay.cand_scores) : nullptr;
   p.S = (float*)(sb + lay.S);
+  L->rows = uses_rows(cfg);
   L->sweep = uses_sweep(cfg);
   L->inplace = L->sweep && (cfg->debug_outputs & 32) && rr_route_sweep_inplace_supported(p);
   L->fused = uses_fused(cfg);

@@ -47,7 +47,8 @@ struct rr_ledger {
   unsigned call_index;                     // layer calls since reset (parity of the force_state slots)
   int timeout_shots;                       // test hook: forced time-outs still to be fired (bit 0
                                            // routing kernel, bit 1 strip rescoring kernel)
-  bool sweep;                              // full routing runs in the two-sweep fused kernel
+  bool rows;                               // full routing runs in the two-threads-per-row kernel
+  bool sweep;                              // ... else in the four-threads-per-row kernel
   bool inplace;                            // relay: challenge test inside the routing kernel
   bool fused;                              // ... else in the streaming fused kernel
   bool dense_rescore;                      // relay rescoring reads the tensor-core score strip
@@ -120,6 +121,9 @@ cudaError_t rr_launch_score_tc(const RRParams& p, const void* qc, const void* kc
 bool rr_route_fused_supported(const RRParams& p);
 cudaError_t rr_launch_route_fused(const RRParams& p, const void* qc, const void* kc,
                                   const int32_t* row_list, int layer, cudaStream_t st);
+bool rr_route_rows_supported(const RRParams& p);
+cudaError_t rr_launch_route_rows(const RRParams& p, const void* qc, const void* kc, const int32_t* row_list,
+                                 int layer, int hooks, cudaStream_t st);   // hooks: as below
 bool rr_route_sweep_supported(const RRParams& p);
 cudaError_t rr_launch_route_sweep(const RRParams& p, const void* qc, const void* kc,
                                   const int32_t* row_list, int layer, int inplace, int hooks,

@@ -43,6 +43,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 constexpr uint32_t kSpinLimit = 1u << 22;
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
                                           volatile uint32_t* abort_flag) {
+#pragma unroll 1
   for (uint32_t it = 0; it < kSpinLimit; ++it) {
     if (mbar_try_wait(bar, parity)) return true;
     if (it > 64) {
@@ -59,6 +60,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity,
 // hardware-defined slice, so this is of the order of a second).
 __device__ __forceinline__ bool mbar_wait_spin(uint64_t* bar, uint32_t parity,
                                                volatile uint32_t* abort_flag) {
+#pragma unroll 1
   for (uint32_t it = 0; it < kSpinLimit; ++it) {
     if (mbar_try_wait(bar, parity)) return true;
     if ((it & 63u) == 63u && *abort_flag) return false;
@@ -74,7 +76,8 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity,
                                                volatile uint32_t* abort_flag, uint32_t ns) {
   bool ok = false;
   if ((threadIdx.x & 31) == 0) {
-    for (uint32_t it = 0; it < kSpinLimit; ++it) {
+  #pragma unroll 1
+  for (uint32_t it = 0; it < kSpinLimit; ++it) {
       if (mbar_try_wait(bar, parity)) { ok = true; break; }
       if (*abort_flag) break;
       __nanosleep(ns);
@@ -92,6 +95,7 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity,
 // issue slots from the warps that share their schedulers.
 __device__ __forceinline__ bool mbar_wait_relaxed(uint64_t* bar, uint32_t parity,
                                                   volatile uint32_t* abort_flag, uint32_t ns) {
+#pragma unroll 1
   for (uint32_t it = 0; it < kSpinLimit; ++it) {
     if (mbar_try_wait(bar, parity)) return true;
     if (*abort_flag) return false;
@@ -121,6 +125,25 @@ __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* t
       ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(z),
         "r"(smem_u32(bar))
       : "memory");
+}
+// A whole tile of rows x d bf16 as d / 64 K-halves of [rows][64] (4-D map of
+// rr_encode_tmap_bf16_tile), issued by a CONVERGED WARP: all 32 lanes call, one elected lane announces
+// `bytes` on the barrier and starts the copy.  Back to back, 8 KB boxes, that takes 180 cycles per
+// copy; from inside a single-lane branch the pair takes 313.
+__device__ __forceinline__ void tma_load_tile_warp(uint32_t smem_dst, const CUtensorMap* tmap, int y, int z,
+                                                   uint64_t* bar, uint32_t bytes) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%5], %6;\n\t"
+      "@e cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%2, %3, %2, %4}], [%5];\n\t}"
+      ::"r"(smem_dst), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(0), "r"(y), "r"(z), "r"(smem_u32(bar)), "r"(bytes)
+      : "memory");
+}
+__device__ __forceinline__ void tma_prefetch_l2_tile(const CUtensorMap* tmap, int y, int z) {
+  asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %1, %3}];"
+               ::"l"(reinterpret_cast<uint64_t>(tmap)), "r"(0), "r"(y), "r"(z) : "memory");
 }
 // The same tile fetched into L2 only (no shared-memory destination, no barrier): hides the
 // DRAM latency of a tile that a later tma_load_3d will ask for.
@@ -231,6 +254,38 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
                : "memory");
 }
 
+// The same two operations issued by a CONVERGED WARP: all 32 lanes call, one elected lane issues (the
+// same one every time, so a commit covers the warp's MMAs).  In warp-uniform control flow the
+// descriptors stay in uniform registers; from inside a single-lane branch every tcgen05.mma costs
+// about 84 cycles of issue whatever its size, here 33 (N = 64) or 65 (N = 128), the tensor pipe's
+// own rate (measured: 512 MMAs back to back, one CTA per SM).
+__device__ __forceinline__ void umma_bf16_ts_warp(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc,
+                                                  uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, e;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+      ::"r"(tmem_d), "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+__device__ __forceinline__ void umma_bf16_warp(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
+                                               uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p, e;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+__device__ __forceinline__ void umma_commit_warp(uint64_t* bar) {
+  asm volatile("{\n\t.reg .pred e;\n\t"
+               "elect.sync _|e, 0xffffffff;\n\t"
+               "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+               ::"r"(smem_u32(bar)) : "memory");
+}
+
 // 32 lanes x 32 consecutive fp32 columns: thread t of the warp gets row (lane base + t).
 // The wait for the asynchronous load sits in the same asm block, so no use of the registers
 // can be scheduled ahead of it.
@@ -292,3 +347,7 @@ __device__ __forceinline__ void tmem_ld_32x64(uint32_t taddr, uint32_t (&a)[32],
 // 128-byte swizzle (entry point fetched from the driver at run time; no libcuda link).
 cudaError_t rr_encode_tmap_bf16_3d(CUtensorMap* out, const void* base, int d, int rows, int planes,
                                    int box_rows);
+// The same tensor as a 4-D map [planes][d / 64][rows][64] with a {64, box_rows, d / 64, 1} box: one
+// copy brings box_rows whole rows, K-half by K-half.
+cudaError_t rr_encode_tmap_bf16_tile(CUtensorMap* out, const void* base, int d, int rows, int planes,
+                                     int box_rows);

@@ -1,0 +1,54 @@
+"""The two-threads-per-row routing kernel at the edges of its dispatch and of its tiles: column
+capacities (keep = k + max(m, 1) at 28 | 29, 48 | 49, 96 | 97), key chunks around the 64-wide tiles
+and the two-tile round of a row's threads, rows that see fewer chunks than they keep, ragged row
+tiles and widths that rule out 16-byte stores."""
+import numpy as np
+import pytest
+import torch
+
+import parity
+from paper_2609_07306_b200 import workload as W
+from paper_2609_07306_b200.ledger import RouteLedger, config_from_workload, device_tensor
+
+pytestmark = pytest.mark.gpu
+
+
+def _w(n_q, n_k, d, k, m, r, causal, **kw):
+    return W.RouteWorkload("edge", 1, 2, n_q, n_k, d, k, m, r, layers=3, anchor_every=100, dtype=W.DTYPE_BF16,
+                           centroids=12, rho=0.2, causal=causal, seed=21, **kw)
+
+
+@pytest.mark.parametrize("k,m", [(20, 8), (20, 9), (32, 16), (33, 16), (47, 0), (16, 32), (64, 32), (65, 32), (3, 1)])
+def test_widths_around_the_column_capacities(k, m):
+    rep = parity.run_teacher_forced(_w(150, 700, 128, k, m, 9, True, causal_offset=550))
+    parity.assert_clean(rep)
+
+
+@pytest.mark.parametrize("n_k", [1, 33, 63, 64, 65, 127, 128, 129, 192, 193, 1025])
+def test_key_chunks_around_the_tiles(n_k):
+    k = min(12, n_k)
+    rep = parity.run_teacher_forced(_w(129, n_k, 64, k, min(8, n_k - k), 5, False))
+    parity.assert_clean(rep)
+    rep = parity.run_teacher_forced(_w(131, n_k, 128, k, 8, 5, True))
+    parity.assert_clean(rep)
+
+
+def test_best_chunks_in_one_threads_tiles():
+    """Scores whose best chunks all lie in even tiles (one thread's share of every row), then in a
+    handful of columns: the bound follows, routes stay exact."""
+    w = _w(128, 1024, 64, 32, 16, 16, False)
+    rng = np.random.default_rng(5)
+    q = rng.standard_normal((2, 128, 64)).astype(np.float32)
+    for boost in (lambda c: (c // 64) % 2 == 0, lambda c: c >= 1024 - 60, lambda c: c % 64 < 4):
+        k = rng.standard_normal((2, 1024, 64)).astype(np.float32)
+        k += np.where(boost(np.arange(1024)), 4.0, 0.0)[None, :, None] * q.mean(axis=1, keepdims=True)
+        qb, kb = (W.f32_to_bf16_bits(x) for x in (q, k))
+        led = RouteLedger(config_from_workload(w))
+        led.route_anchor(device_tensor(qb), device_tensor(kb), 0)
+        torch.cuda.synchronize()
+        assert led.status() == 0
+        s = np.einsum("pid,pjd->pij", W.bf16_bits_to_f32(qb).astype(np.float64), W.bf16_bits_to_f32(kb).astype(np.float64))
+        want = np.sort(np.argsort(-s, axis=2)[:, :, :32], axis=2).reshape(-1, 32)
+        got = led.routes.cpu().numpy()
+        assert (got == want).all(axis=1).mean() > 0.999      # (float64 against fp32: near-ties only)
+        led.close()
