@@ -90,7 +90,7 @@ rescore_dense_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q,
   const uint32_t xch_base = (bm_base + tcpipe::BM * pitch * 4u + 15u) & ~15u;
   const uint32_t sc_base = xch_base + 3u * PITCH;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0), lane = tid & 31;
   const int tiles_m = p.tiles_per_problem;
   const int prob = blockIdx.x % p.P, tm = tiles_m - 1 - blockIdx.x / p.P;   // heaviest first
   const int tile_id = prob * tiles_m + tm;
@@ -138,9 +138,9 @@ rescore_dense_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q,
   const int n_tiles = pipe.num_tiles(p);
 
   if (warp == 0) {
-    if (lane == 0) pipe.producer(&tmap_k, prob, n_tiles, &tmap_q, tm);
+    pipe.producer(&tmap_k, prob, n_tiles, &tmap_q, tm);
   } else if (warp == 1) {
-    if (lane == 0) pipe.mma_issuer(n_tiles, true);
+    pipe.mma_issuer(n_tiles, true);
   } else {
     // a warp may only read the TMEM lanes 32*(warp % 4) ...: warps 2-5 take the first COLS
     // columns of their quarter's rows, warps 6-9 the rest

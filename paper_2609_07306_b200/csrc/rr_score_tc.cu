@@ -31,7 +31,7 @@ score_tc_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   ScorePipe<D> pipe;
   pipe.carve(smem_raw);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const int tiles_m = p.tiles_per_problem;
   const int prob = blockIdx.x / tiles_m, tm = blockIdx.x % tiles_m;
 
@@ -44,9 +44,9 @@ score_tc_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   const int n_tiles = pipe.num_tiles(p);
 
   if (warp == 0) {
-    if (lane == 0) pipe.producer(&tmap_k, prob, n_tiles);
+    pipe.producer(&tmap_k, prob, n_tiles);
   } else if (warp == 1) {
-    if (lane == 0) pipe.mma_issuer(n_tiles);
+    pipe.mma_issuer(n_tiles);
   } else {
     // ===== epilogue: one thread per query row =====
     const int quarter = warp & 3;                         // TMEM lane quarter of this warp

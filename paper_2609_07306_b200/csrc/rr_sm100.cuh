@@ -141,6 +141,17 @@ __device__ __forceinline__ void tma_load_tile_warp(uint32_t smem_dst, const CUte
       ::"r"(smem_dst), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(0), "r"(y), "r"(z), "r"(smem_u32(bar)), "r"(bytes)
       : "memory");
 }
+__device__ __forceinline__ void tma_load_3d_warp(uint32_t smem_dst, const CUtensorMap* tmap, int x, int y, int z,
+                                                 uint64_t* bar, uint32_t bytes) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\t"
+      "elect.sync _|e, 0xffffffff;\n\t"
+      "@e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%5], %6;\n\t"
+      "@e cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes "
+      "[%0], [%1, {%2, %3, %4}], [%5];\n\t}"
+      ::"r"(smem_dst), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)), "r"(bytes)
+      : "memory");
+}
 __device__ __forceinline__ void tma_prefetch_l2_tile(const CUtensorMap* tmap, int y, int z) {
   asm volatile("cp.async.bulk.prefetch.tensor.4d.L2.global.tile [%0, {%1, %2, %1, %3}];"
                ::"l"(reinterpret_cast<uint64_t>(tmap)), "r"(0), "r"(y), "r"(z) : "memory");

@@ -1,8 +1,8 @@
 // The producer side of the tensor-core score kernels: one CTA owns BM = 128 query rows of one
 // problem and streams score tiles S[128 rows, BN key chunks] into a ring of TMEM accumulators.
-//   warp 0, lane 0 : TMA producer -- Kc tiles (bf16, 128-byte swizzle, no multicast) into a ring
+//   warp 0         : TMA producer -- Kc tiles (bf16, 128-byte swizzle, no multicast) into a ring
 //                    of B_STAGES shared-memory stages
-//   warp 1, lane 0 : issues tcgen05.mma (M=128, N=BN, K=16; d/16 steps per tile) into a ring of
+//   warp 1         : issues tcgen05.mma (M=128, N=BN, K=16; d/16 steps per tile) into a ring of
 //                    ACC_STAGES TMEM accumulators of BN columns and commits to mbarriers
 //   consumers      : CONSUMERS threads (one or more per row); wait on acc_full[stage], read
 //                    TMEM with tcgen05.ld, then arrive on acc_empty[stage]
@@ -69,9 +69,10 @@ struct Pipe {
       ctl->row[tid] = row; ctl->slot[tid] = slot;
     }
     if (tid == 0) {
-      for (int s = 0; s < B_STAGES; ++s) { mbar_init(&ctl->full[s], 1); mbar_init(&ctl->empty[s], 1); }
+      // (one arrival per announced K-half)
+      for (int s = 0; s < B_STAGES; ++s) { mbar_init(&ctl->full[s], KHALVES); mbar_init(&ctl->empty[s], 1); }
       for (int s = 0; s < ACC_STAGES; ++s) { mbar_init(&ctl->acc_full[s], 1); mbar_init(&ctl->acc_empty[s], CONSUMERS); }
-      mbar_init(&ctl->a_full, 1);
+      mbar_init(&ctl->a_full, KHALVES);
       mbar_init(&ctl->drain, 1);
       ctl->abort_flag = 0;
       mbar_fence_init();
@@ -109,61 +110,63 @@ struct Pipe {
     return (vmax + BN - 1) / BN;
   }
 
+  // Whole, converged warps run the two roles (see umma_bf16_ts_warp / tma_load_3d_warp).
   __device__ __forceinline__ void producer(const CUtensorMap* tmap_k, int prob, int n_tiles,
                                            const CUtensorMap* tmap_q = nullptr, int tm = 0) {
     volatile uint32_t* abort_flag = &ctl->abort_flag;
+    const uint32_t a_addr = smem_u32(sA), b_addr = smem_u32(sB);
     if (tmap_q) {                                         // rows past n_q are zero-filled
-      mbar_expect_tx(&ctl->a_full, A_BYTES);
 #pragma unroll
       for (int h = 0; h < KHALVES; ++h)
-        tma_load_3d(sA + h * A_HALF, tmap_q, h * 64, tm * BM, prob, &ctl->a_full);
+        tma_load_3d_warp(a_addr + h * A_HALF, tmap_q, h * 64, tm * BM, prob, &ctl->a_full, A_HALF);
     }
-    int issued = 0;
-    for (int t = 0; t < n_tiles; ++t) {
+    int t = 0;
+#pragma unroll 1
+    for (; t < n_tiles; ++t) {
       const int s = t % B_STAGES; const uint32_t ph = (t / B_STAGES) & 1;
-      if (!mbar_wait_relaxed(&ctl->empty[s], ph ^ 1, abort_flag, 400)) break;
-      mbar_expect_tx(&ctl->full[s], B_BYTES);
+      if (!__all_sync(0xFFFFFFFFu, mbar_wait_spin(&ctl->empty[s], ph ^ 1, abort_flag))) break;
 #pragma unroll
       for (int h = 0; h < KHALVES; ++h)
-        tma_load_3d(sB + s * B_BYTES + h * B_HALF, tmap_k, h * 64, t * BN, prob, &ctl->full[s]);
-      ++issued;
+        tma_load_3d_warp(b_addr + s * B_BYTES + h * B_HALF, tmap_k, h * 64, t * BN, prob, &ctl->full[s], B_HALF);
     }
     // do not leave while copies into this CTA's shared memory may still be in flight
-    for (int t = max(0, issued - B_STAGES); t < issued; ++t) {
-      const int s = t % B_STAGES; const uint32_t ph = (t / B_STAGES) & 1;
-      for (uint32_t it = 0; it < kSpinLimit && !mbar_try_wait(&ctl->full[s], ph); ++it) __nanosleep(64);
-    }
+#pragma unroll 1
+    for (int u = max(0, t - B_STAGES); u < t; ++u)
+#pragma unroll 1
+      for (uint32_t it = 0; it < kSpinLimit && !mbar_try_wait(&ctl->full[u % B_STAGES], (u / B_STAGES) & 1); ++it) __nanosleep(64);
     if (tmap_q)
+#pragma unroll 1
       for (uint32_t it = 0; it < kSpinLimit && !mbar_try_wait(&ctl->a_full, 0); ++it) __nanosleep(64);
+    __syncwarp();
   }
 
   __device__ __forceinline__ void mma_issuer(int n_tiles, bool q_by_tma = false) {
     volatile uint32_t* abort_flag = &ctl->abort_flag;
-    if (q_by_tma && !mbar_wait(&ctl->a_full, 0, abort_flag)) return;
+    const uint32_t tmem_u = __shfl_sync(0xFFFFFFFFu, ctl->tmem_base, 0);
     constexpr uint32_t idesc = umma_idesc_bf16(BM, BN);
-    const uint32_t a_addr = smem_u32(sA);
-    const uint32_t tmem_base = ctl->tmem_base;
+    const uint64_t a_desc = umma_desc_k_sw128(smem_u32(sA)), b_desc = umma_desc_k_sw128(smem_u32(sB));
+    if (q_by_tma && !__all_sync(0xFFFFFFFFu, mbar_wait(&ctl->a_full, 0, abort_flag))) return;
+#pragma unroll 1
     for (int t = 0; t < n_tiles; ++t) {
       const int s = t % B_STAGES; const uint32_t ph = (t / B_STAGES) & 1;
       const int as = t % ACC_STAGES; const uint32_t aph = (t / ACC_STAGES) & 1;
-      if (!mbar_wait_relaxed(&ctl->acc_empty[as], aph ^ 1, abort_flag, 400)) break;
-      if (!mbar_wait_relaxed(&ctl->full[s], ph, abort_flag, 100)) break;
+      if (!__all_sync(0xFFFFFFFFu, mbar_wait_spin(&ctl->acc_empty[as], aph ^ 1, abort_flag))) break;
+      if (!__all_sync(0xFFFFFFFFu, mbar_wait_spin(&ctl->full[s], ph, abort_flag))) break;
       tc_fence_after();
-      const uint32_t b_addr = smem_u32(sB + s * B_BYTES);
 #pragma unroll
-      for (int k = 0; k < KSTEPS; ++k) {
-        const uint32_t a_off = (k >> 2) * A_HALF + (k & 3) * 32;
-        const uint32_t b_off = (k >> 2) * B_HALF + (k & 3) * 32;
-        umma_bf16(tmem_base + as * BN, umma_desc_k_sw128(a_addr + a_off),
-                  umma_desc_k_sw128(b_addr + b_off), idesc, k > 0 ? 1u : 0u);
-      }
-      umma_commit(&ctl->empty[s]);        // smem stage reusable once these MMAs have read it
-      umma_commit(&ctl->acc_full[as]);    // accumulator ready for the consumers
+      for (int k = 0; k < KSTEPS; ++k)
+        umma_bf16_warp(tmem_u + as * BN, a_desc + (uint64_t)((k >> 2) * (A_HALF >> 4) + (k & 3) * 2),
+                       b_desc + (uint64_t)(s * (B_BYTES >> 4) + (k >> 2) * (B_HALF >> 4) + (k & 3) * 2), idesc,
+                       k > 0 ? 1u : 0u);
+      umma_commit_warp(&ctl->empty[s]);        // smem stage reusable once these MMAs have read it
+      umma_commit_warp(&ctl->acc_full[as]);    // accumulator ready for the consumers
     }
     // TMEM must not be freed while an MMA can still write to it: after a wait that gave up the
     // consumers no longer vouch for that, so the issuer waits (bounded) for its own MMAs
-    umma_commit(&ctl->drain);
+    umma_commit_warp(&ctl->drain);
+#pragma unroll 1
     for (uint32_t it = 0; it < kSpinLimit && !mbar_try_wait(&ctl->drain, 0); ++it) __nanosleep(64);
+    __syncwarp();
   }
 
   // Consumer side of one tile: returns false (for the whole warp) if the wait gave up.
