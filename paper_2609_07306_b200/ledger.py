@@ -9,6 +9,52 @@ from . import binding as B
 from .workload import DTYPE_BF16, RouteWorkload
 
 _TORCH_DT = {"i32": torch.int32, "f32": torch.float32, "u8": torch.uint8, "i64": torch.int64}
+_BYTES = {"i32": 4, "f32": 4, "u8": 1, "i64": 8}
+
+
+def _raw_stream(device: torch.device) -> int:
+    """The current stream's handle (without building a torch.cuda.Stream object per call)."""
+    return torch._C._cuda_getCurrentRawStream(device.index)
+
+
+class _Views:
+    """Zero-copy tensors over the library's device pointers, made once each: the buffers and the
+    pointers stay the same for the ledger's life.  One as_strided per view over a typed alias of
+    the buffer it lies in."""
+
+    def _init_views(self):
+        self._view_cache = {}
+        self._aliases = {}
+
+    def _alias(self, which: int, kind: str) -> torch.Tensor:
+        a = self._aliases.get((which, kind))
+        if a is None:
+            buf = (self.ledger_buf, self.scratch_buf)[which]
+            a = self._aliases[(which, kind)] = buf[:buf.numel() // 8 * 8].view(_TORCH_DT[kind])
+        return a
+
+    def _view(self, name: str, kind: str, shape):
+        t = self._view_cache.get(name)
+        if t is not None:
+            return t
+        ptr = getattr(self._views, name)
+        if not ptr:
+            return None
+        n = 1
+        for x in shape:
+            n *= x
+        for which, buf in enumerate((self.ledger_buf, self.scratch_buf)):
+            off = ptr - buf.data_ptr()
+            if 0 <= off and off + n * _BYTES[kind] <= buf.numel():
+                strides, step = [], 1
+                for x in reversed(shape):
+                    strides.insert(0, step)
+                    step *= x
+                alias = self._alias(which, kind)
+                t = alias.as_strided(shape, strides, off // _BYTES[kind])
+                self._view_cache[name] = t
+                return t
+        raise RuntimeError(f"view {name} lies outside the ledger buffers")
 
 
 def config_from_workload(w: RouteWorkload, debug_outputs: bool = False,
@@ -32,7 +78,7 @@ def config_from_workload(w: RouteWorkload, debug_outputs: bool = False,
                        force_permille=int(w.force_permille), force_max_run=int(w.force_max_run))
 
 
-class RouteLedger:
+class RouteLedger(_Views):
     """Owns the two device buffers of one ledger and exposes the C calls as methods."""
 
     def __init__(self, cfg: B.rr_config, device: str = "cuda:0"):
@@ -40,6 +86,8 @@ class RouteLedger:
             raise RuntimeError("RouteLedger needs a CUDA device (there is no CPU path)")
         self.cfg = cfg
         self.device = torch.device(device)
+        if self.device.index is None:
+            self.device = torch.device("cuda", torch.cuda.current_device())
         lb, sb = B.rr_workspace_bytes(cfg)
         with torch.cuda.device(self.device):
             self.ledger_buf = torch.empty(lb + 256, dtype=torch.uint8, device=self.device)
@@ -53,6 +101,8 @@ class RouteLedger:
         self.sw = cfg.m + cfg.r + (cfg.global_sentinels & 1) + ((cfg.global_sentinels >> 1) & 1)
         self.c = cfg.k + self.sw
         self._views = B.rr_ledger_views(self.handle)
+        self._init_views()
+        self._anchor, self._relay = B.lib().rr_route_anchor, B.lib().rr_route_relay
         self.reset()
 
     # -- lifetime ------------------------------------------------------------------------
@@ -69,17 +119,21 @@ class RouteLedger:
             pass
 
     def _stream(self) -> int:
-        return torch.cuda.current_stream(self.device).cuda_stream
+        return _raw_stream(self.device)
 
     # -- calls -----------------------------------------------------------------------------
     def reset(self):
         B.rr_ledger_reset(self.handle, self._stream())
 
     def route_anchor(self, qc: torch.Tensor, kc: torch.Tensor, layer: int):
-        B.rr_route_anchor(self.handle, qc.data_ptr(), kc.data_ptr(), layer, self._stream())
+        rc = self._anchor(self.handle, qc.data_ptr(), kc.data_ptr(), layer, _raw_stream(self.device))
+        if rc != B.RR_OK:
+            raise B.RouteRelayError(rc, "rr_route_anchor")
 
     def route_relay(self, qc: torch.Tensor, kc: torch.Tensor, layer: int):
-        B.rr_route_relay(self.handle, qc.data_ptr(), kc.data_ptr(), layer, self._stream())
+        rc = self._relay(self.handle, qc.data_ptr(), kc.data_ptr(), layer, _raw_stream(self.device))
+        if rc != B.RR_OK:
+            raise B.RouteRelayError(rc, "rr_route_relay")
 
     def route_layer_host(self, host_qc: torch.Tensor, host_kc: torch.Tensor,
                          dev_qc: torch.Tensor, dev_kc: torch.Tensor, layer: int,
@@ -105,20 +159,7 @@ class RouteLedger:
     def status(self) -> int:
         return B.rr_ledger_status(self.handle, self._stream())
 
-    # -- views (zero-copy torch tensors over the library's device pointers) ---------------
-    def _view(self, name: str, kind: str, shape):
-        ptr = getattr(self._views, name)
-        if not ptr:
-            return None
-        n = int(np.prod(shape))
-        dt = _TORCH_DT[kind]
-        nbytes = n * torch.empty((), dtype=dt).element_size()
-        for buf in (self.ledger_buf, self.scratch_buf):
-            off = ptr - buf.data_ptr()
-            if 0 <= off and off + nbytes <= buf.numel():
-                return buf[off:off + nbytes].view(dt).view(*shape)
-        raise RuntimeError(f"view {name} lies outside the ledger buffers")
-
+    # -- views ------------------------------------------------------------------------------
     @property
     def routes(self): return self._view("routes", "i32", (self.rows, self.cfg.k))
     @property
@@ -193,6 +234,8 @@ class _BucketLedger(RouteLedger):
         self.sw = cfg.m + cfg.r + (cfg.global_sentinels & 1) + ((cfg.global_sentinels >> 1) & 1)
         self.c = cfg.k + self.sw
         self._views = B.rr_ledger_views(handle)
+        self._init_views()
+        self._anchor, self._relay = B.lib().rr_route_anchor, B.lib().rr_route_relay
 
     def close(self):
         self.handle = None
@@ -206,6 +249,8 @@ class BucketSet:
         if not torch.cuda.is_available():
             raise RuntimeError("BucketSet needs a CUDA device (there is no CPU path)")
         self.cfg, self.device = cfg, torch.device(device)
+        if self.device.index is None:
+            self.device = torch.device("cuda", torch.cuda.current_device())
         self.order, n_buckets, lb, sb = B.rr_bucket_plan(cfg, widths)
         with torch.cuda.device(self.device):
             self.ledger_buf = torch.empty(lb + 256, dtype=torch.uint8, device=self.device)
@@ -228,7 +273,7 @@ class BucketSet:
         self.reset()
 
     def _stream(self) -> int:
-        return torch.cuda.current_stream(self.device).cuda_stream
+        return _raw_stream(self.device)
 
     def reset(self):
         B.rr_bucket_set_reset(self.handle, self._stream())
@@ -264,5 +309,5 @@ def attend_token_ranges(ranges: torch.Tensor, n_q: int, q: torch.Tensor, keys: t
     out = torch.empty((rows, q.shape[1]), dtype=torch.float32, device=q.device)
     B.rr_attend_token_ranges(ranges.data_ptr(), rows, slots, n_q, q.data_ptr(), keys.data_ptr(),
                              values.data_ptr(), keys.shape[1], q.shape[1], dtype, float(scale),
-                             out.data_ptr(), torch.cuda.current_stream(q.device).cuda_stream)
+                             out.data_ptr(), _raw_stream(q.device))
     return out
