@@ -84,6 +84,13 @@ RRParams shape_params(const rr_config* cfg) {
 // Which kernel routes rows.  Two threads per row with two CTAs per SM (rr_route_rows.cu) wherever
 // its shape limits hold; the relay in place (debug bit 5) exists in the four-threads-per-row kernel
 // only; the streaming kernel takes wider routes (and debug bit 4), the two-pass path the rest.
+// fp32 inputs are scored, tested and routed in one kernel per row tile, unless the two-pass or the
+// gathered form is asked for (10 problems of 384 x 192, c = 48: relay 135 + 7 + 9 us for gathered test,
+// GEMM and selection).
+bool uses_f32(const rr_config* cfg) {
+  return !(cfg->debug_outputs & (2 | 4)) && rr_route_f32_supported(shape_params(cfg));
+}
+
 bool uses_sweep(const rr_config* cfg) {
   return (cfg->debug_outputs & 32) && !(cfg->debug_outputs & (2 | 16)) && rr_route_sweep_supported(shape_params(cfg));
 }
@@ -118,14 +125,14 @@ Layout make_layout(const rr_config* c) {
   L.refresh_rows = o;    o = align_up(o + rows * 4);
   L.refresh_count = o;   o = align_up(o + 4);
   L.problem_offsets = o; o = align_up(o + (P + 1) * 4);
-  L.tile_counts = o;     o = align_up(o + tiles * 4);
+  L.tile_counts = o;     o = align_up(o + 2 * tiles * 4);
   L.counters = o;        o = align_up(o + RR_NUM_COUNTERS * 8);
   L.status = o;          o = align_up(o + 4);
   L.force_state = o;     o = align_up(o + 8 * 4);
   L.token_ranges = o;    o = align_up(o + (c->chunk_tokens > 0 ? rows * c->k * 8 : 0));
   L.cand_scores = o;     o = align_up(o + ((c->debug_outputs & 1) ? rows * cw * 4 : 0));
   // score rows are only materialised by the two-pass path
-  L.S = o;               o = align_up(o + (uses_fused(c) || uses_sweep(c) || uses_rows(c) ? 0 : rows * (size_t)c->n_k * 4));
+  L.S = o;               o = align_up(o + (uses_fused(c) || uses_sweep(c) || uses_rows(c) || uses_f32(c) ? 0 : rows * (size_t)c->n_k * 4));
   L.scratch_total = o;
   return L;
 }
@@ -153,6 +160,7 @@ int route_layer(rr_ledger* L, const void* qc, const void* kc, int layer, bool an
   RRParams p = L->p;
   p.force_in = p.force_stats + 2 * (L->call_index & 1u);
   p.force_out = p.force_stats + 2 * ((L->call_index + 1u) & 1u);
+  if (L->call_index & 1u) { int32_t* t = p.tile_counts; p.tile_counts = p.tile_counts_next; p.tile_counts_next = t; }
   ++L->call_index;
   // LAUNCH(kind, call): enqueue one kernel, bracketed by events while profiling
 #define LAUNCH(kind, call)                                                         \
@@ -168,7 +176,9 @@ int route_layer(rr_ledger* L, const void* qc, const void* kc, int layer, bool an
   if (anchor) {
     // Section 4.1: the anchor builds the state from a complete chunk-score matrix.
     LAUNCH(RR_KIND_ANCHOR_FILL, rr_launch_anchor_fill(p, L->dense_pairs_per_layer, st));
-    if (L->rows) {
+    if (L->f32) {
+      LAUNCH(RR_KIND_ROUTE_FUSED, rr_launch_route_f32(p, qc, kc, 1, layer, st));
+    } else if (L->rows) {
       LAUNCH(RR_KIND_ROUTE_FUSED, rr_launch_route_rows(p, qc, kc, nullptr, layer, sweep_hooks(L), st));
     } else if (L->sweep) {
       LAUNCH(RR_KIND_ROUTE_FUSED, rr_launch_route_sweep(p, qc, kc, nullptr, layer, 0,
@@ -192,6 +202,12 @@ int route_layer(rr_ledger* L, const void* qc, const void* kc, int layer, bool an
                                                         sweep_hooks(L), st));
       LAUNCH(RR_KIND_COMPACT, rr_launch_compact(p, L->dense_pairs_per_layer, st));
       LAUNCH(RR_KIND_SENTINELS, rr_launch_sentinels(p, p.refresh_rows, layer, st));
+      if (p.chunk_tokens > 0) LAUNCH(RR_KIND_EXPAND, rr_launch_expand(p, 0, st));
+      return RR_OK;
+    }
+    if (L->f32) {
+      LAUNCH(RR_KIND_ROUTE_FUSED, rr_launch_route_f32(p, qc, kc, 0, layer, st));
+      LAUNCH(RR_KIND_COMPACT, rr_launch_compact(p, L->dense_pairs_per_layer, st));
       if (p.chunk_tokens > 0) LAUNCH(RR_KIND_EXPAND, rr_launch_expand(p, 0, st));
       return RR_OK;
     }
@@ -285,6 +301,7 @@ int rr_ledger_init(const rr_config* cfg, void* dev_ledger, size_t ledger_bytes,
   p.refresh_count = (int32_t*)(sb + lay.refresh_count);
   p.problem_offsets = (int32_t*)(sb + lay.problem_offsets);
   p.tile_counts = (int32_t*)(sb + lay.tile_counts);
+  p.tile_counts_next = p.tile_counts + p.n_tiles;     // (swapped every other call, route_layer)
   p.counters = (unsigned long long*)(sb + lay.counters);
   p.status = (uint32_t*)(sb + lay.status);
   p.force_stats = (int32_t*)(sb + lay.force_state);
@@ -294,6 +311,7 @@ int rr_ledger_init(const rr_config* cfg, void* dev_ledger, size_t ledger_bytes,
   p.token_ranges = cfg->chunk_tokens > 0 ? (int32_t*)(sb + lay.token_ranges) : nullptr;
   p.cand_scores = (cfg->debug_outputs & 1) ? (float*)(sb + lay.cand_scores) : nullptr;
   p.S = (float*)(sb + lay.S);
+  L->f32 = uses_f32(cfg);
   L->rows = uses_rows(cfg);
   L->sweep = uses_sweep(cfg);
   L->inplace = L->sweep && (cfg->debug_outputs & 32) && rr_route_sweep_inplace_supported(p);

@@ -25,7 +25,8 @@ struct RRParams {
   int32_t* routes; int32_t* sentinels; int32_t* ages; float* kth; float* margin;
   // per-layer outputs and scratch
   uint8_t* flags; float* alpha; float* beta; float* tau;
-  int32_t* refresh_rows; int32_t* refresh_count; int32_t* problem_offsets; int32_t* tile_counts;
+  int32_t* refresh_rows; int32_t* refresh_count; int32_t* problem_offsets;
+  int32_t* tile_counts; int32_t* tile_counts_next;   // flagged rows per row tile of this call / the next one
   int32_t* token_ranges; float* cand_scores;
   unsigned long long* counters; uint32_t* status;
   float* S;                                // [rows, n_k] score rows of the two-pass path
@@ -51,6 +52,7 @@ struct rr_ledger {
   bool sweep;                              // ... else in the four-threads-per-row kernel
   bool inplace;                            // relay: challenge test inside the routing kernel
   bool fused;                              // ... else in the streaming fused kernel
+  bool f32;                                // fp32 inputs: test and routing in one kernel
   bool dense_rescore;                      // relay rescoring reads the tensor-core score strip
   unsigned long long dense_pairs_per_layer;
   // benchmark-only per-kernel timing
@@ -112,10 +114,33 @@ __device__ __forceinline__ bool rr_challenge(const RRParams& p, int g, float alp
   return flag;
 }
 
+// ---- programmatic dependent launch ---------------------------------------------------------
+// A layer is a chain of short kernels.  Launched with rr_launch_pdl, a kernel may start while its
+// predecessor in the stream drains: it sets itself up and calls rr_pdl_wait() before it reads
+// anything an earlier kernel writes (inputs included: they may come from the caller's kernels).
+// rr_pdl_trigger() lets the successor start; every kernel calls it AFTER its own wait, so that
+// whatever ran before a kernel has finished by the time the kernel after it starts.  Both are no-ops
+// in a kernel launched the ordinary way.  Every path through such a kernel waits.
+__device__ __forceinline__ void rr_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void rr_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <class... P, class... A>
+inline cudaError_t rr_launch_pdl(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem; cfg.stream = st; cfg.attrs = &attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ---- launchers (one per .cu file) -------------------------------------------------------
 // All return cudaError_t from the launch; all are asynchronous on `st`.
 cudaError_t rr_launch_score_simt(const RRParams& p, const void* qc, const void* kc,
                                  const int32_t* row_list, cudaStream_t st);
+bool rr_route_f32_supported(const RRParams& p);
+cudaError_t rr_launch_route_f32(const RRParams& p, const void* qc, const void* kc, int anchor, int layer,
+                                cudaStream_t st);
 cudaError_t rr_launch_score_tc(const RRParams& p, const void* qc, const void* kc,
                                const int32_t* row_list, cudaStream_t st);
 bool rr_route_fused_supported(const RRParams& p);

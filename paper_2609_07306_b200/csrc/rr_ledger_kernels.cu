@@ -23,6 +23,9 @@ compact_kernel(RRParams p, unsigned long long dense_pairs) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tile_id = blockIdx.x;
   const int prob = tile_id / p.tiles_per_problem, tile = tile_id % p.tiles_per_problem;
+  rr_pdl_wait();
+  rr_pdl_trigger();
+  if (tid == 0) p.tile_counts_next[tile_id] = 0;       // (for kernels that add to the counts)
 
   // Forced anchor (Section 3.2, policy of rr_config.force_permille): the previous tested relay
   // flagged so many rows that this call routes every row.  The tile does what the anchor's fill
@@ -103,6 +106,9 @@ compact_kernel(RRParams p, unsigned long long dense_pairs) {
 __global__ void anchor_fill_kernel(RRParams p, unsigned long long dense_pairs) {
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   const float qnan = __int_as_float(0x7fc00000);
+  rr_pdl_wait();
+  rr_pdl_trigger();
+  if (g < p.n_tiles) p.tile_counts_next[g] = 0;
   if (g < p.rows) {
     p.flags[g] = 1;
     p.refresh_rows[g] = g;
@@ -130,6 +136,8 @@ __global__ void __launch_bounds__(256)
 expand_kernel(RRParams p, int is_anchor) {
   const int lane = threadIdx.x & 31;
   const int g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  rr_pdl_wait();
+  rr_pdl_trigger();
   if (g >= p.rows) return;
   if (!(is_anchor || p.flags[g] != 0)) return;       // stable row: ranges unchanged
   const int32_t* route = p.routes + (size_t)g * p.k;
@@ -210,7 +218,7 @@ __global__ void reset_kernel(RRParams p) {
     p.flags[e] = 0; p.alpha[e] = 0.f; p.beta[e] = 0.f; p.refresh_rows[e] = -1;
   }
   for (size_t e = tid; e <= (size_t)p.P; e += stride) p.problem_offsets[e] = 0;
-  for (size_t e = tid; e < (size_t)p.n_tiles; e += stride) p.tile_counts[e] = 0;
+  for (size_t e = tid; e < (size_t)p.n_tiles; e += stride) { p.tile_counts[e] = 0; p.tile_counts_next[e] = 0; }
   if (p.token_ranges)
     for (size_t e = tid; e < (size_t)p.rows * p.k * 2; e += stride) p.token_ranges[e] = -1;
   if (tid < RR_NUM_COUNTERS) p.counters[tid] = 0;
@@ -221,25 +229,25 @@ __global__ void reset_kernel(RRParams p) {
 }  // namespace
 
 cudaError_t rr_launch_compact(const RRParams& p, unsigned long long dense_pairs, cudaStream_t st) {
-  compact_kernel<<<p.n_tiles, RR_ROW_TILE, 0, st>>>(p, dense_pairs);
+  const cudaError_t e = rr_launch_pdl(compact_kernel, p.n_tiles, RR_ROW_TILE, 0, st, p, dense_pairs);
   rr_count_launch();
-  return cudaPeekAtLastError();
+  return e;
 }
 
 cudaError_t rr_launch_anchor_fill(const RRParams& p, unsigned long long dense_pairs,
                                   cudaStream_t st) {
   const int n = p.rows > p.P + 1 ? p.rows : p.P + 1;
-  anchor_fill_kernel<<<(n + 255) / 256, 256, 0, st>>>(p, dense_pairs);
+  const cudaError_t e = rr_launch_pdl(anchor_fill_kernel, (n + 255) / 256, 256, 0, st, p, dense_pairs);
   rr_count_launch();
-  return cudaPeekAtLastError();
+  return e;
 }
 
 cudaError_t rr_launch_expand(const RRParams& p, int is_anchor, cudaStream_t st) {
   const int wpb = 8;
   const size_t smem = p.coalesce ? (size_t)wpb * p.k * sizeof(int32_t) : 0;
-  expand_kernel<<<(p.rows + wpb - 1) / wpb, wpb * 32, smem, st>>>(p, is_anchor);
+  const cudaError_t e = rr_launch_pdl(expand_kernel, (p.rows + wpb - 1) / wpb, wpb * 32, smem, st, p, is_anchor);
   rr_count_launch();
-  return cudaPeekAtLastError();
+  return e;
 }
 
 cudaError_t rr_launch_reset(const RRParams& p, cudaStream_t st) {
