@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(NT, 2)
 rescore_dense_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q,
                      const __grid_constant__ CUtensorMap tmap_k, int words, int force_timeout) {
   using P = tcpipe::Pipe<D, BN, B_STAGES, ACC_STAGES, NCONS>;
+  rr_pdl_wait();
   if (p.force_threshold > 0 && p.force_in[0] > 0) return;   // forced anchor: nothing is tested
   extern __shared__ uint8_t smem_raw[];
   P pipe;
@@ -135,6 +136,7 @@ rescore_dense_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q,
   load16(pre1_is1 ? ptr1 : ptr0, pre1_s0, pre1_is1 ? n1 : n0, pre1);
 
   pipe.setup(p, nullptr, &tmap_k, nullptr, prob, tm, 0, p.n_q, NT, &tmap_q);
+  rr_pdl_trigger();                             // (not before: the successor takes TMEM, too)
   const int n_tiles = pipe.num_tiles(p);
 
   if (warp == 0) {
@@ -325,14 +327,9 @@ cudaError_t rr_launch_rescore_dense(const RRParams& p, const void* qc, const voi
     return cudaSuccess;
   });
   if (e != cudaSuccess) return e;
-  const int grid = p.n_tiles;
-  if (p.d == 128) {
-    if (prior) rescore_dense_kernel<128, true><<<grid, NT, smem, st>>>(p, tmap_q, tmap, words, force_timeout);
-    else rescore_dense_kernel<128, false><<<grid, NT, smem, st>>>(p, tmap_q, tmap, words, force_timeout);
-  } else {
-    if (prior) rescore_dense_kernel<64, true><<<grid, NT, smem, st>>>(p, tmap_q, tmap, words, force_timeout);
-    else rescore_dense_kernel<64, false><<<grid, NT, smem, st>>>(p, tmap_q, tmap, words, force_timeout);
-  }
+  auto kernel = p.d == 128 ? (prior ? rescore_dense_kernel<128, true> : rescore_dense_kernel<128, false>)
+                           : (prior ? rescore_dense_kernel<64, true> : rescore_dense_kernel<64, false>);
+  e = rr_launch_pdl(kernel, p.n_tiles, NT, smem, st, p, tmap_q, tmap, words, force_timeout);
   rr_count_launch();
-  return cudaPeekAtLastError();
+  return e;
 }

@@ -274,16 +274,6 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   constexpr int TILE = BN * D * 2;
   static_assert(STAGES >= 2 && STAGES <= ACC_STAGES, "see produce()");
   constexpr int M = CAP / 2;                               // entries per half column
-  // a relay call that the forced-anchor policy turned into full routing has the identity list:
-  // take the anchor's path (consecutive rows, no gathers through the list)
-  const bool forced_call = row_list_arg && p.force_threshold > 0 && p.force_in[0] > 0;
-  // A refresh list that holds nearly every row (high drift) is served the same way, with the
-  // rows that are not on it masked out: gathering 7/8 of the rows through the list costs more
-  // than sweeping the missing eighth for nothing (results per row are the same either way).
-  const bool dense_refresh = row_list_arg && !forced_call &&
-                             (long long)(*p.refresh_count) * 8 >= (long long)p.rows * 7;
-  const int32_t* __restrict__ row_list = (forced_call || dense_refresh) ? nullptr : row_list_arg;
-  const bool force_hard = hooks & 1, force_timeout = hooks & 2;      // test hooks
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* sB = smem;                                      // Kc ring; after the sweeps: keys, bitmap
@@ -296,6 +286,30 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
 #ifdef RR_PHASE_TIMING
   const long long cta_t0_ = clock64();
 #endif
+  if (tid == 0) {
+    for (int s = 0; s < STAGES; ++s) mbar_init(&ctl->full[s], 1);
+    for (int s = 0; s < ACC_STAGES; ++s) {
+      mbar_init(&ctl->acc_full[s], 1);
+      mbar_init(&ctl->acc_empty[s], SEL_WARPS / TPR);      // one arrival per warp that reads the tile
+    }
+    mbar_init(&ctl->drain, 1);
+    ctl->abort_flag = 0;
+    ctl->hard_n = 0;
+    mbar_fence_init();
+  }
+  // The predecessor writes the refresh list; at an anchor it only fills in book-keeping, and the
+  // inputs have been complete since it started (see rr_launch_pdl).
+  if (row_list_arg) rr_pdl_wait();
+  // a relay call that the forced-anchor policy turned into full routing has the identity list:
+  // take the anchor's path (consecutive rows, no gathers through the list)
+  const bool forced_call = row_list_arg && p.force_threshold > 0 && p.force_in[0] > 0;
+  // A refresh list that holds nearly every row (high drift) is served the same way, with the
+  // rows that are not on it masked out: gathering 7/8 of the rows through the list costs more
+  // than sweeping the missing eighth for nothing (results per row are the same either way).
+  const bool dense_refresh = row_list_arg && !forced_call &&
+                             (long long)(*p.refresh_count) * 8 >= (long long)p.rows * 7;
+  const int32_t* __restrict__ row_list = (forced_call || dense_refresh) ? nullptr : row_list_arg;
+  const bool force_hard = hooks & 1, force_timeout = hooks & 2;      // test hooks
   // Row tiles are handed out heaviest first (under the causal mask the last tile of a problem
   // walks the most key chunks), so the tail of the grid is made of the short ones.
   const int tiles_m = p.tiles_per_problem;
@@ -303,7 +317,7 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
 
   int seg_lo = 0, seg_hi = p.n_q;
   if (row_list) { seg_lo = p.problem_offsets[prob]; seg_hi = p.problem_offsets[prob + 1]; }
-  if (tm * BM >= seg_hi - seg_lo) return;                  // nothing to do (uniform per CTA)
+  if (tm * BM >= seg_hi - seg_lo) { if (!row_list_arg) rr_pdl_wait(); return; }   // nothing to do (uniform per CTA)
 
   // row of the CTA's tile -> query row of the problem and global row id; -1 = no row
   auto locate = [&](int rr, int& row_out, int& g_out) {
@@ -338,18 +352,10 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
     }
   }
   if (is_sel && j == 0) { ctl->row[r] = row; ctl->hard_slot[r] = -1; }
-  if (tid == 0) {
-    for (int s = 0; s < STAGES; ++s) mbar_init(&ctl->full[s], 1);
-    for (int s = 0; s < ACC_STAGES; ++s) {
-      mbar_init(&ctl->acc_full[s], 1);
-      mbar_init(&ctl->acc_empty[s], SEL_WARPS / TPR);      // one arrival per warp that reads the tile
-    }
-    mbar_init(&ctl->drain, 1);
-    ctl->abort_flag = 0;
-    ctl->hard_n = 0;
-    mbar_fence_init();
+  if (warp == 1) {
+    tmem_alloc(&ctl->tmem_base, TMEM_COLS);
+    rr_pdl_trigger();                                      // (not before: the successor takes TMEM, too)
   }
-  if (warp == 1) tmem_alloc(&ctl->tmem_base, TMEM_COLS);
   // The Kc loads depend on nothing but the number of key tiles (from the tile's last row: rows
   // ascend inside a tile), and the ring's stages are all free: the producer fills the ring before
   // the CTA's first barrier, while the Qc rows are on their way.
@@ -833,6 +839,7 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
     tmem_dealloc(tmem_base, TMEM_COLS);
   }
   if (tid == 0 && ctl->abort_flag) atomicOr(p.status, RR_STATUS_TIMEOUT);
+  if (!row_list_arg) rr_pdl_wait();                        // complete only after the predecessor is
 }
 
 // ---- configurations ------------------------------------------------------------------------------
@@ -903,8 +910,8 @@ cudaError_t rr_launch_route_rows(const RRParams& p, const void* qc, const void* 
     return cudaSuccess;
   });
   if (e != cudaSuccess) return e;
-  kernel_of(p.d, pl.variant)<<<p.n_tiles, NT, pl.smem, st>>>(p, (const __nv_bfloat16*)qc, tmap, row_list,
-                                                            (uint32_t)layer, hooks, pl.ring_bytes, 2 * 148);
+  e = rr_launch_pdl(kernel_of(p.d, pl.variant), p.n_tiles, NT, pl.smem, st, p, (const __nv_bfloat16*)qc, tmap, row_list,
+                    (uint32_t)layer, hooks, pl.ring_bytes, 2 * 148);
   rr_count_launch();
-  return cudaPeekAtLastError();
+  return e;
 }
