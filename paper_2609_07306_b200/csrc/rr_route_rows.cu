@@ -35,8 +35,8 @@
 // by binary search over the two sorted halves; route and near-miss ids are gathered, ordered by
 // chunk id in registers and leave with 16-byte stores.  The second thread of the row then draws
 // the sentinels against the row's bitmap of excluded chunks.
-// Rows the fast path cannot finish exactly (the column overflowed, scores out of order within
-// the fixed-point resolution, equal scores across a cut)
+// Rows the fast path cannot finish exactly (the column overflowed, three scores out of order
+// within the fixed-point resolution)
 // are handed to an exact slow path: one more sweep stores their complete score rows in shared
 // memory, and a warp per row runs the radix select of the two-pass path.  Every mbarrier wait is
 // bounded.
@@ -62,16 +62,13 @@ constexpr uint32_t WORD_PITCH = BM * 4;            // [word][row] areas
 struct Ctl {
   uint64_t full[MAX_STAGES], acc_full[ACC_STAGES], acc_empty[ACC_STAGES], drain;
   uint32_t tmem_base, abort_flag, hard_n, pad_;
-  int row[BM];                          // query row of the problem, -1 = no row
-  float bound[TPR][BM], top[TPR][BM];   // per thread of a row: bound from its share, largest maximum
-  int8_t shift[BM];                     // how far the shares move (towards thread 0 if positive)
   uint8_t cnt[TPR][BM];                 // survivors per thread
-  uint8_t cut[TPR][BM];                 // entries of the first half-column in the top k / top k + m
-  uint8_t bad[TPR][BM];                 // a thread of the row asks for the slow path
+  uint8_t cut[TPR][BM];                 // entries of the first half column in the top k / top k + m; bit 7: slow path
   uint8_t hard_rows[BM];                // rows handed to the slow path, in registration order
   int8_t hard_slot[BM];                 // position of a row in hard_rows, -1 = none
 };
-constexpr int CTL_BYTES = 4096;
+constexpr int CTL_BYTES = 1024;
+constexpr int MAIL = 20;                // slot of a half column through which its thread gets the other's messages
 static_assert(sizeof(Ctl) <= CTL_BYTES, "control block too large");
 
 __device__ __forceinline__ uint32_t lds32(uint32_t a) {
@@ -265,7 +262,7 @@ __device__ unsigned long long g_rows_phase[32];
 #endif
 
 // NG: classes of a thread's tiles (128 NG groups of columns per row); CAP: entries per row.
-template <int D, int NG, int CAP, int CTAS, int STAGES>
+template <int D, int NG, int CAP, int CTAS, int STAGES, int ROUNDS>
 __global__ void __launch_bounds__(NT, CTAS)
 route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
                   const __grid_constant__ CUtensorMap tmap_k, const int32_t* __restrict__ row_list_arg,
@@ -274,8 +271,8 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   constexpr int TILE = BN * D * 2;
   static_assert(STAGES >= 2 && STAGES <= ACC_STAGES, "see produce()");
   constexpr int M = CAP / 2;                               // entries per half column
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  extern __shared__ __align__(1024) uint8_t smem_raw[];    // (checked below: the swizzle needs it)
+  uint8_t* smem = smem_raw;
   uint8_t* sB = smem;                                      // Kc ring; after the sweeps: keys, bitmap
   Ctl* ctl = (Ctl*)(smem + ring_bytes);
   uint8_t* s_col = (uint8_t*)ctl + CTL_BYTES;              // [CAP][BM] entries
@@ -296,6 +293,11 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
     ctl->abort_flag = 0;
     ctl->hard_n = 0;
     mbar_fence_init();
+  }
+  if ((smem_u32(smem) & 1023u) != 0u) {                    // reported like a wait that gave up
+    if (tid == 0) atomicOr(p.status, RR_STATUS_TIMEOUT);
+    rr_pdl_wait();
+    return;
   }
   // The predecessor writes the refresh list; at an anchor it only fills in book-keeping, and the
   // inputs have been complete since it started (see rr_launch_pdl).
@@ -351,7 +353,7 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
       qv[4 * i] = t.x; qv[4 * i + 1] = t.y; qv[4 * i + 2] = t.z; qv[4 * i + 3] = t.w;
     }
   }
-  if (is_sel && j == 0) { ctl->row[r] = row; ctl->hard_slot[r] = -1; }
+  if (is_sel && j == 0) ctl->hard_slot[r] = -1;
   if (warp == 1) {
     tmem_alloc(&ctl->tmem_base, TMEM_COLS);
     rr_pdl_trigger();                                      // (not before: the successor takes TMEM, too)
@@ -556,12 +558,18 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
       share0 = min(g0, max(share0, T - g1));
       int share = j == 0 ? share0 : T - share0;
       float bound = share_bound(share);
-      ctl->bound[j][r] = bound;
-      ctl->top[j][r] = fmaxf(A(0), B(0));
+      // messages: word 0 of the other thread's mail slot = this thread's bound, word 1 = the shift
+      const uint32_t mail_in = col + (uint32_t)(j * M + MAIL) * SLOT_PITCH, mail_out = col + (uint32_t)((1 - j) * M + MAIL) * SLOT_PITCH;
+      float top = fmaxf(A(0), B(0));
+      sts32(mail_out, __float_as_uint(bound));
 #pragma unroll 1
-      for (int round = 0; round < 2; ++round) {
+      for (int round = 0; round < ROUNDS; ++round) {
         quarter_sync(quarter);
-        const float other = ctl->bound[1 - j][r];
+        const float other = ldsf(mail_in);
+        if (round == 0) {                                    // (the other list is still there)
+          const uint32_t w = lds32(col + (uint32_t)((1 - j) * M) * SLOT_PITCH);
+          top = fmaxf(top, fmaxf(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u)));
+        }
         // the thread with the higher bound counts its maxima at or above the other one's and takes
         // half of the surplus
         int ca = 0, cb = 0;
@@ -571,25 +579,29 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
           cb += B(cb + s - 1) >= other ? s : 0;
         }
         ca += A(ca) >= other ? 1 : 0; cb += B(cb) >= other ? 1 : 0;   // ca, cb <= 31 here
-        const int shift = max(0, (ca + cb - share) >> 1);
-        if (bound > other) ctl->shift[r] = (int8_t)(j == 0 ? shift : -shift);
-        if (bound == other && j == 0) ctl->shift[r] = 0;
+        int shift = max(0, (ca + cb - share) >> 1);
+        if (j == 1) shift = -shift;
+        if (bound > other) sts32(mail_out + 4u, (uint32_t)shift);
         quarter_sync(quarter);
-        share0 = min(min(g0, T), max(share0 + (int)ctl->shift[r], max(T - g1, 0)));
+        if (bound < other) shift = (int)lds32(mail_in + 4u);
+        if (bound == other) shift = 0;
+        share0 = min(min(g0, T), max(share0 + shift, max(T - g1, 0)));
         share = j == 0 ? share0 : T - share0;
         bound = share_bound(share);
-        ctl->bound[j][r] = bound;
+        sts32(mail_out, __float_as_uint(bound));
       }
-      // the lists are done with: the half column is cleared (empty slots read as -inf in the sort)
+      // the lists are done with: the half column is cleared (empty slots read as -inf in the sort), the
+      // mail slot once its last message has been read
 #pragma unroll
-      for (int e = 0; e < M; ++e) sts64(col + (uint32_t)(j * M + e) * SLOT_PITCH, 0xff800000u, 0u);
+      for (int e = 0; e < M; ++e)
+        if (e != MAIL) sts64(col + (uint32_t)(j * M + e) * SLOT_PITCH, 0xff800000u, 0u);
       quarter_sync(quarter);
-      tau = fminf(bound, ctl->bound[1 - j][r]);
+      tau = fminf(bound, ldsf(mail_in));
+      sts64(mail_in, 0xff800000u, 0u);
       // a maximum is a score with its low half cut off, i.e. moved towards zero: a negative bound is
       // lowered by one bf16 step, a positive top raised by one
       const uint32_t tb = __float_as_uint(tau);
       if ((tb & 0x80000000u) && tb != 0xff800000u) tau = __uint_as_float(tb + 0x10000u);
-      float top = fmaxf(ctl->top[0][r], ctl->top[1][r]);
       if (top >= 0.f) top = __uint_as_float(__float_as_uint(top + 0.f) + 0x10000u);
       scale = __fdividef(1.0f - 1.0f / 2097152.0f, top - tau);
       if (!(top > tau && scale < 1e30f)) scale = 0.f;        // nothing to tell apart
@@ -636,20 +648,50 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
     bool bad = have && (n > CAP || n < T);                   // (too few only after a wait gave up)
     const uint32_t half = col + (uint32_t)(j * M) * SLOT_PITCH;
     {
+      // equal keys keep the ascending chunk ids of their thread: slots ascend with the ids in thread
+      // 0's half, descend in thread 1's
+      const uint32_t flip = j == 0 ? 255u : 0u;
       uint32_t key[M];
 #pragma unroll
       for (int i = 0; i < M; ++i)
-        key[i] = fixed_bits(ldsf(half + (uint32_t)i * SLOT_PITCH), tau, scale) * 256u + (uint32_t)i;
+        key[i] = fixed_bits(ldsf(half + (uint32_t)i * SLOT_PITCH), tau, scale) * 256u + (uint32_t)(j == 0 ? 255 - i : i);
       OESort<0, pow2_at_least(M), DescPos, M>::run(key);
       uint32_t es[M], ei[M];
 #pragma unroll
-      for (int i = 0; i < M; ++i) lds64(half + (key[i] & 255u) * SLOT_PITCH, es[i], ei[i]);
-      bool wrong = false;                                    // two scores the keys could not tell apart
+      for (int i = 0; i < M; ++i) lds64(half + ((key[i] & 255u) ^ flip) * SLOT_PITCH, es[i], ei[i]);
+      bool wrong = false;
 #pragma unroll
-      for (int i = 0; i + 1 < M; ++i) wrong |= __uint_as_float(es[i]) < __uint_as_float(es[i + 1]);
-      bad |= have && wrong;
+      for (int i = 0; i + 1 < M; ++i)
+        wrong |= !(__uint_as_float(es[i]) > __uint_as_float(es[i + 1]) || (es[i] == es[i + 1] && ei[i] <= ei[i + 1]));
 #pragma unroll
       for (int i = 0; i < M; ++i) sts64(half + (uint32_t)i * SLOT_PITCH, es[i], ei[i]);
+      // Keys that agree in all 23 bits leave their two entries in slot order: about one row in 5000
+      // has such a pair.  One pass of exchanges repairs pairs; what is out of order after it (a run of
+      // three) is left to the slow path.
+      if (__any_sync(FULL, have && wrong)) {
+        wrong = false;
+        uint32_t s0, i0;
+        lds64(half, s0, i0);
+        float above = pinf;
+        uint32_t above_id = 0;
+        auto follows = [&](uint32_t sc, uint32_t id) {                 // does not rank before its predecessor
+          wrong |= __uint_as_float(sc) > above || (__uint_as_float(sc) == above && id < above_id);
+          above = __uint_as_float(sc); above_id = id;
+        };
+#pragma unroll 1
+        for (int i = 1; i < M; ++i) {
+          uint32_t s1, i1;
+          lds64(half + (uint32_t)i * SLOT_PITCH, s1, i1);
+          const bool ok = __uint_as_float(s0) > __uint_as_float(s1) || (s0 == s1 && i0 <= i1);
+          const uint32_t fs = ok ? s0 : s1, fi = ok ? i0 : i1;         // goes to slot i - 1
+          sts64(half + (uint32_t)(i - 1) * SLOT_PITCH, fs, fi);
+          follows(fs, fi);
+          s0 = ok ? s1 : s0; i0 = ok ? i1 : i0;
+        }
+        sts64(half + (uint32_t)(M - 1) * SLOT_PITCH, s0, i0);
+        follows(s0, i0);
+      }
+      bad |= have && wrong;
     }
     // the bitmap of excluded chunks starts empty (the Kc ring is idle once the last tile of sweep 2
     // has been consumed)
@@ -660,25 +702,40 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
     quarter_sync(quarter);
 
     // ===== cuts: thread 0 rank k, thread 1 rank k + m ====================================================
-    auto HA = [&](int i) -> float { return ldsf(col + (uint32_t)i * SLOT_PITCH); };
-    auto HB = [&](int i) -> float { return ldsf(col + (uint32_t)(M + i) * SLOT_PITCH); };
     const int rank = j == 0 ? kk : p.m > 0 ? T : kk;         // m = 0: no near-miss sentinels
     {
-      const int a = rank_split<M>(min(rank, CAP), HA, HB), b = rank - a;
-      const float la = HA(max(a - 1, 0)), lb = HB(min(max(b - 1, 0), M - 1)), xa = HA(min(a, M - 1)), xb = HB(min(max(b, 0), M - 1));
-      const float last_in = fminf(a > 0 ? la : pinf, b > 0 ? lb : pinf);
-      const float first_out = fmaxf(a < M ? xa : ninf, b < M ? xb : ninf);
-      bad |= have && !(last_in > first_out);                 // equal scores straddle the cut
+      // entry a of the first half ranks before entry b of the second: higher score, or equal score and
+      // smaller chunk id
+      int lo = max(0, rank - M), hi = min(rank, M);
+#pragma unroll 1
+      for (int s = 1; s <= M; s *= 2) {
+        const int mid = (lo + hi) >> 1;
+        uint32_t sa, ia, sb, ib;
+        lds64(col + (uint32_t)min(mid, M - 1) * SLOT_PITCH, sa, ia);
+        lds64(col + (uint32_t)(M + min(max(rank - mid - 1, 0), M - 1)) * SLOT_PITCH, sb, ib);
+        const float fa = __uint_as_float(sa), fb = __uint_as_float(sb);
+        const bool more = fa > fb || (fa == fb && ia < ib), step_ = lo < hi;
+        lo = step_ && more ? mid + 1 : lo;
+        hi = step_ && !more ? mid : hi;
+      }
+      const int a = lo, b = rank - a;
+      auto score = [&](int slot) -> float { return ldsf(col + (uint32_t)slot * SLOT_PITCH); };
       if (force_hard && have && g % 5 == 0) bad = true;      // test hook: exercise the slow path
-      ctl->cut[j][r] = (uint8_t)a;
-      ctl->bad[j][r] = bad;
-      if (j == 0 && have && !bad) {                          // (overwritten by the slow path if it takes the row)
-        p.kth[g] = last_in;
-        p.margin[g] = v > kk ? last_in - first_out : pinf;
+      ctl->cut[j][r] = (uint8_t)(a | (bad ? 128 : 0));
+      if (j == 0) {
+        const float la = score(max(a - 1, 0)), lb = score(M + min(max(b - 1, 0), M - 1));
+        const float xa = score(min(a, M - 1)), xb = score(M + min(max(b, 0), M - 1));
+        const float last_in = fminf(a > 0 ? la : pinf, b > 0 ? lb : pinf);
+        const float first_out = fmaxf(a < M ? xa : ninf, b < M ? xb : ninf);
+        if (have && !bad) {                                  // (overwritten by the slow path if it takes the row)
+          p.kth[g] = last_in;
+          p.margin[g] = v > kk ? last_in - first_out : pinf;
+        }
       }
     }
     quarter_sync(quarter);
-    const bool hard = ctl->bad[0][r] | ctl->bad[1][r];
+    const int a_k = ctl->cut[0][r] & 127, a_d = ctl->cut[1][r] & 127;
+    const bool hard = ((ctl->cut[0][r] | ctl->cut[1][r]) & 128) != 0;
     const bool go = have && !hard;
     if (j == 0 && hard) {
       const uint32_t idx = atomicAdd(&ctl->hard_n, 1u);
@@ -691,7 +748,6 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
     const int n_excl = p.m > 0 ? T : kk;                     // route + near-miss ids of the row
     int32_t* const sent = p.sentinels + (size_t)g * p.sw;
     {
-      const int a_k = ctl->cut[0][r], a_d = ctl->cut[1][r];
       const int e0 = j == 0 ? 0 : a_k, n0 = j == 0 ? a_k : a_d - a_k;
       const int e1 = M + (j == 0 ? 0 : kk - a_k), n1 = j == 0 ? kk - a_k : (n_excl - a_d) - (kk - a_k);
       const int width = j == 0 ? p.k : p.m;
@@ -813,10 +869,10 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
       uint32_t* scratch = (uint32_t*)s_col + (size_t)hard_slots * nk_words * 32 + sw * (256 + nk_words);
       for (int hs = sw; hs < hard_slots && done + hs < n_hard; hs += SEL_WARPS) {
         const int rr = ctl->hard_rows[done + hs];
-        const int hv = rr_valid_count(ctl->row[rr], p.n_k, p.causal, p.causal_offset);
+        const int hg = row_list ? row_list[seg_lo + tm * BM + rr] : prob * p.n_q + tm * BM + rr;
+        const int hv = rr_valid_count(hg - prob * p.n_q, p.n_k, p.causal, p.causal_offset);
         const uint32_t* keys = (const uint32_t*)s_col + (size_t)hs * nk_words * 32;
-        warptopk::route_row(p, keys, scratch, scratch + 256, row_list ? row_list[seg_lo + tm * BM + rr] : prob * p.n_q + ctl->row[rr],
-                            hv, layer, lane);
+        warptopk::route_row(p, keys, scratch, scratch + 256, hg, hv, layer, lane);
         __syncwarp();
       }
     }
@@ -845,9 +901,10 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
 // ---- configurations ------------------------------------------------------------------------------
 // keep = k + max(m, 1) decides how many entries a row's column needs: the bound lets 1.05-1.25 keep
 // scores pass while keep is at most 3/8 of the groups (mean / largest of 10^5 random rows: keep 24,
-// 1024 chunks: 26.7 / 37; keep 48, 576 and 1024 chunks: 57.8 / 80 and 58.9 / 80; with 256 groups,
-// keep 96, 2048 chunks: 119 / 140).  A row that needs more takes the slow path (7 in 100,000 at
-// keep 48).  Beyond 48 the column and the second set of maxima leave room for one CTA per SM.
+// 1024 chunks: 27.1 / 40; keep 48, 576 and 1024 chunks: 57.8 / 80 and 58.9 / 80; with 256 groups,
+// keep 96, 2048 chunks: 119 / 140).  A row that needs more takes the slow path (fewer than 3 in
+// 10^6 at keep 48; a column of 76 entries let 7 in 10^5 through, and the CTA that meets one runs
+// 12 us longer: 289 instead of 265 us on 2048 CTAs).  Beyond 48 the column and the second set of maxima leave room for one CTA per SM.
 struct Plan { int variant, ring_bytes; size_t smem; };
 
 bool plan(const RRParams& p, Plan& out) {
@@ -855,7 +912,7 @@ bool plan(const RRParams& p, Plan& out) {
   if (p.dtype != RR_BF16 || (p.d != 64 && p.d != 128) || p.n_k > RR_MAX_NK) return false;
   int cap;
   if (keep <= 28) { out.variant = 0; cap = 48; }
-  else if (keep <= 48) { out.variant = 1; cap = 76; }
+  else if (keep <= 48) { out.variant = 1; cap = 80; }
   else if (keep <= 96) { out.variant = 2; cap = 152; }
   else return false;
   const int words = (p.n_k + 31) / 32;
@@ -863,15 +920,15 @@ bool plan(const RRParams& p, Plan& out) {
   int ring = stages * BN * p.d * 2;
   if (ring < words * (int)WORD_PITCH) ring = words * (int)WORD_PITCH;
   out.ring_bytes = (ring + 1023) / 1024 * 1024;
-  out.smem = 1024 + (size_t)out.ring_bytes + CTL_BYTES + (size_t)cap * SLOT_PITCH;
+  out.smem = (size_t)out.ring_bytes + CTL_BYTES + (size_t)cap * SLOT_PITCH;
   return out.smem <= 227 * 1024;
 }
 
 typedef void (*Kernel)(RRParams, const __nv_bfloat16*, const CUtensorMap, const int32_t*, uint32_t, int, int, int);
 Kernel kernel_of(int d, int variant) {
   static const Kernel table[2][3] = {
-      {route_rows_kernel<64, 1, 48, 2, 3>, route_rows_kernel<64, 1, 76, 2, 3>, route_rows_kernel<64, 2, 152, 1, 3>},
-      {route_rows_kernel<128, 1, 48, 2, 3>, route_rows_kernel<128, 1, 76, 2, 2>, route_rows_kernel<128, 2, 152, 1, 3>}};
+      {route_rows_kernel<64, 1, 48, 2, 3, 1>, route_rows_kernel<64, 1, 80, 2, 3, 2>, route_rows_kernel<64, 2, 152, 1, 3, 1>},
+      {route_rows_kernel<128, 1, 48, 2, 3, 1>, route_rows_kernel<128, 1, 80, 2, 2, 2>, route_rows_kernel<128, 2, 152, 1, 3, 1>}};
   return table[d == 128 ? 1 : 0][variant];
 }
 
