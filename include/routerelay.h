@@ -310,7 +310,8 @@ int rr_bucket_set_count(const rr_bucket_set* S);                 /* number of bu
 int rr_bucket_set_info(const rr_bucket_set* S, int32_t b, rr_bucket_info* out);
 rr_ledger* rr_bucket_set_ledger(rr_bucket_set* S, int32_t b);    /* borrowed; for rr_ledger_views */
 int rr_bucket_set_reset(rr_bucket_set* S, void* stream);
-/* One layer for all buckets, enqueued on `stream` bucket after bucket.  qc / kc: device,
+/* One layer for all buckets, ordered on `stream` like any other call: the buckets run side by side
+ * on streams of the set that start from `stream` and are joined to it.  qc / kc: device,
  * bucket-major [P, n_q, d] / [P, n_k, d].  is_anchor != 0: anchor layer, else relay layer
  * (RR_ERR_STATE before the first anchor). */
 int rr_bucket_route_layer(rr_bucket_set* S, const void* qc, const void* kc, int32_t layer,
