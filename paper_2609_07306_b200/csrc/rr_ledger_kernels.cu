@@ -130,19 +130,12 @@ __global__ void anchor_fill_kernel(RRParams p, unsigned long long dense_pairs) {
 }
 
 // ---- token ranges of the rows that were re-routed -------------------------------------------
-// One warp per row: ids are ranked by counting (they are distinct), chunk j -> [j*T, (j+1)*T),
-// ascending chunk id, (-1,-1) for empty slots.
-__global__ void __launch_bounds__(256)
-expand_kernel(RRParams p, int is_anchor) {
-  const int lane = threadIdx.x & 31;
-  const int g = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  rr_pdl_wait();
-  rr_pdl_trigger();
-  if (g >= p.rows) return;
-  if (!(is_anchor || p.flags[g] != 0)) return;       // stable row: ranges unchanged
+// Chunk j -> [j*T, (j+1)*T), ascending chunk id, (-1,-1) for empty slots.  General form, one warp per
+// row: ids that are out of order are ranked by counting (they are distinct).
+__device__ void expand_row(const RRParams& p, int g, int lane, int32_t* srt) {
   const int32_t* route = p.routes + (size_t)g * p.k;
   int32_t* out = p.token_ranges + (size_t)g * p.k * 2;
-  // rows written by the fused routing kernel are already in ascending chunk id with the empty
+  // rows written by the routing kernels are already in ascending chunk id with the empty
   // slots last: their ranges are a plain map of the row (8-byte stores)
   bool ordered = true;
   for (int s = lane; s < p.k; s += 32) {
@@ -153,8 +146,6 @@ expand_kernel(RRParams p, int is_anchor) {
   if (p.coalesce) {
     // the row's ids in ascending order (empty slots last) into shared memory, then one range
     // per run of consecutive ids: a run's first id writes its start, its last id its end
-    extern __shared__ int32_t s_sorted[];
-    int32_t* srt = s_sorted + (threadIdx.x >> 5) * p.k;
     for (int s = lane; s < p.k; s += 32) srt[s] = all_ordered ? route[s] : -1;
     __syncwarp();
     if (!all_ordered) {
@@ -182,6 +173,7 @@ expand_kernel(RRParams p, int is_anchor) {
       base += __popc(starts);
     }
     for (int s = base + lane; s < p.k; s += 32) { out[2 * s] = -1; out[2 * s + 1] = -1; }
+    __syncwarp();
     return;
   }
   if (all_ordered) {
@@ -206,6 +198,49 @@ expand_kernel(RRParams p, int is_anchor) {
     }
   }
   for (int s = n_valid + lane; s < p.k; s += 32) { out[2 * s] = -1; out[2 * s + 1] = -1; }
+}
+
+// A warp takes EXPAND_ROWS rows, so that several loads are in flight before the first store: a row of
+// up to 64 ids is one 8-byte load per lane, checked for order with one shuffle, and one 16-byte store
+// per lane (the plain map).  Bound by DRAM: 100 MB per layer of 131072 rows at k = 64.
+constexpr int EXPAND_ROWS = 4, EXPAND_WARPS = 8;
+__host__ __device__ __forceinline__ bool expand_by_row(const RRParams& p) { return p.coalesce || p.k > 64 || (p.k & 1); }
+__global__ void __launch_bounds__(EXPAND_WARPS * 32)
+expand_kernel(RRParams p, int is_anchor) {
+  extern __shared__ int32_t s_sorted[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  rr_pdl_wait();
+  rr_pdl_trigger();
+  int32_t* const srt = s_sorted + warp * p.k;
+  if (expand_by_row(p)) {
+    const int g = blockIdx.x * EXPAND_WARPS + warp;
+    if (g < p.rows && (is_anchor || p.flags[g] != 0)) expand_row(p, g, lane, srt);   // (stable row: ranges unchanged)
+    return;
+  }
+  const int g0 = (blockIdx.x * EXPAND_WARPS + warp) * EXPAND_ROWS;
+  const int s = 2 * lane, T = p.chunk_tokens;
+  int2 id[EXPAND_ROWS];
+  bool on[EXPAND_ROWS];
+#pragma unroll
+  for (int u = 0; u < EXPAND_ROWS; ++u) {
+    on[u] = g0 + u < p.rows && (is_anchor || p.flags[g0 + u] != 0);
+    id[u] = make_int2(-1, -1);
+    if (on[u] && s < p.k) id[u] = *reinterpret_cast<const int2*>(p.routes + (size_t)(g0 + u) * p.k + s);
+  }
+#pragma unroll
+  for (int u = 0; u < EXPAND_ROWS; ++u) {
+    if (!on[u]) continue;                              // (uniform)
+    const int prev = __shfl_up_sync(FULL, id[u].y, 1);
+    const bool ok = (lane == 0 || id[u].x < 0 || (prev >= 0 && prev < id[u].x)) &&
+                    (id[u].y < 0 || (id[u].x >= 0 && id[u].x < id[u].y));
+    if (!__all_sync(FULL, ok)) { expand_row(p, g0 + u, lane, srt); continue; }
+    if (s < p.k) {
+      int4 o = make_int4(-1, -1, -1, -1);
+      if (id[u].x >= 0) { o.x = id[u].x * T; o.y = o.x + T; }
+      if (id[u].y >= 0) { o.z = id[u].y * T; o.w = o.z + T; }
+      *reinterpret_cast<int4*>(p.token_ranges + ((size_t)(g0 + u) * p.k + s) * 2) = o;
+    }
+  }
 }
 
 __global__ void reset_kernel(RRParams p) {
@@ -243,9 +278,10 @@ cudaError_t rr_launch_anchor_fill(const RRParams& p, unsigned long long dense_pa
 }
 
 cudaError_t rr_launch_expand(const RRParams& p, int is_anchor, cudaStream_t st) {
-  const int wpb = 8;
-  const size_t smem = p.coalesce ? (size_t)wpb * p.k * sizeof(int32_t) : 0;
-  const cudaError_t e = rr_launch_pdl(expand_kernel, (p.rows + wpb - 1) / wpb, wpb * 32, smem, st, p, is_anchor);
+  const int rows_per_block = EXPAND_WARPS * (expand_by_row(p) ? 1 : EXPAND_ROWS);
+  const size_t smem = p.coalesce ? (size_t)EXPAND_WARPS * p.k * sizeof(int32_t) : 0;
+  const cudaError_t e = rr_launch_pdl(expand_kernel, (p.rows + rows_per_block - 1) / rows_per_block, EXPAND_WARPS * 32,
+                                      smem, st, p, is_anchor);
   rr_count_launch();
   return e;
 }
