@@ -212,10 +212,11 @@ int route_layer(rr_ledger* L, const void* qc, const void* kc, int layer, bool an
       return RR_OK;
     }
     // Section 4.2: rescoring + flags, prefix-sum compaction, refresh of the listed rows.
-    if (L->dense_rescore) {
+    if (L->rows_rescore || L->dense_rescore) {
       const int shot = (L->timeout_shots >> 1) & 1;     // test hook: one forced time-out
       L->timeout_shots &= ~2;
-      LAUNCH(RR_KIND_RESCORE_DENSE, rr_launch_rescore_dense(p, qc, kc, shot, /*prior=*/L->fused, st));
+      if (L->rows_rescore) LAUNCH(RR_KIND_RESCORE_DENSE, rr_launch_rescore_rows(p, qc, kc, shot, st));
+      else LAUNCH(RR_KIND_RESCORE_DENSE, rr_launch_rescore_dense(p, qc, kc, shot, st));
     }
     else LAUNCH(RR_KIND_RESCORE, rr_launch_rescore(p, qc, kc, st));
     LAUNCH(RR_KIND_COMPACT, rr_launch_compact(p, L->dense_pairs_per_layer, st));
@@ -316,7 +317,11 @@ int rr_ledger_init(const rr_config* cfg, void* dev_ledger, size_t ledger_bytes,
   L->sweep = uses_sweep(cfg);
   L->inplace = L->sweep && (cfg->debug_outputs & 32) && rr_route_sweep_inplace_supported(p);
   L->fused = uses_fused(cfg);
-  L->dense_rescore = !(cfg->debug_outputs & 4) && rr_rescore_dense_supported(p);
+  // Both rescoring kernels read the score strip; the one that also computes the old candidates' floor
+  // (a third masked pass over every score) runs where the streaming kernel starts from it.
+  const bool strip = !(cfg->debug_outputs & 4);
+  L->rows_rescore = strip && !L->fused && rr_rescore_rows_supported(p);
+  L->dense_rescore = strip && L->fused && rr_rescore_dense_supported(p);
   *out = L;
   return RR_OK;
 }

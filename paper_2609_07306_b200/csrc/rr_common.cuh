@@ -53,7 +53,8 @@ struct rr_ledger {
   bool inplace;                            // relay: challenge test inside the routing kernel
   bool fused;                              // ... else in the streaming fused kernel
   bool f32;                                // fp32 inputs: test and routing in one kernel
-  bool dense_rescore;                      // relay rescoring reads the tensor-core score strip
+  bool rows_rescore;                       // relay rescoring reads the tensor-core score strip
+  bool dense_rescore;                      // ... and leaves a bound for the streaming kernel
   unsigned long long dense_pairs_per_layer;
   // benchmark-only per-kernel timing
   bool profiling = false;
@@ -161,9 +162,12 @@ cudaError_t rr_launch_sentinels(const RRParams& p, const int32_t* row_list, int 
                                 cudaStream_t st);
 cudaError_t rr_launch_rescore(const RRParams& p, const void* qc, const void* kc,
                               cudaStream_t st);
+bool rr_rescore_rows_supported(const RRParams& p);
+cudaError_t rr_launch_rescore_rows(const RRParams& p, const void* qc, const void* kc, int force_timeout,
+                                   cudaStream_t st);
 bool rr_rescore_dense_supported(const RRParams& p);
 cudaError_t rr_launch_rescore_dense(const RRParams& p, const void* qc, const void* kc,
-                                    int force_timeout, bool prior, cudaStream_t st);
+                                    int force_timeout, cudaStream_t st);
 // compact / anchor_fill also advance the ages and the cumulative counters of the layer
 cudaError_t rr_launch_compact(const RRParams& p, unsigned long long dense_pairs, cudaStream_t st);
 cudaError_t rr_launch_anchor_fill(const RRParams& p, unsigned long long dense_pairs,

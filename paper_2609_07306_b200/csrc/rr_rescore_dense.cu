@@ -1,23 +1,18 @@
-// Candidate rescoring + challenge test (Section 3.2, Eq. 5) on the TENSOR CORES.
+// Candidate rescoring + challenge test (Section 3.2, Eq. 5) on the tensor cores, with a bound for the
+// refresh: used where the streaming kernel (rr_route_fused.cu) routes.  rr_rescore_rows.cu is the
+// same test without the bound, which no other kernel reads.
 //
-// The gathered kernel (rr_rescore.cu) fetches c Kc rows per query row and multiplies them on
-// the FP32 ALUs: no operand is reused, so it moves c*d*2 bytes per row through L2 and is an
-// order of magnitude slower on this machine than computing the whole score strip with
-// tcgen05.mma.  This variant does the latter: the same kind of tile pipeline as the fused
-// routing kernel produces S[128 rows, 64 chunks] tiles in TMEM, and the threads of a row pick
-// out the scores of the row's candidates:
+// The tile pipeline of rr_tc_pipeline.cuh produces S[128 rows, 64 chunks] tiles in TMEM:
 //   * at start the two threads of a row turn its ledger row into a bitmap in shared memory (two
-//     planes encoding route / near-miss / random sentinel, one plane per thread), reading the
-//     ids with 16-byte loads and setting bits with grouped read-modify-writes;
+//     planes encoding route / near-miss / random sentinel, one plane per thread);
 //   * per tile a thread reads its share of the row's scores from TMEM and takes masked minima /
 //     maxima under the tile's bitmap words: alpha = min over route bits, beta = max over
 //     sentinel bits, floor = min over route and near-miss bits (the refresh's warm-start
 //     threshold).
-// Scores are bit-identical to the ones the fused routing kernel computes (same instruction
+// Scores are bit-identical to the ones the streaming kernel computes (same instruction
 // sequence on the same operands), so the floor needs no safety margin.
 // Outputs are those of the gathered kernel: flags, alpha, beta, tau, per-tile flagged counts,
-// work counters (the candidate pairs are still charged as c per row: that is what the method
-// evaluates; that the hardware computes the strip is an implementation matter).
+// work counters.
 #include "rr_tc_pipeline.cuh"
 
 using namespace sm100;
@@ -69,11 +64,9 @@ __device__ unsigned long long g_rd_phase[8];
 // of a warp fall into 32 different banks whenever each thread touches a word of its own row).
 // Two planes encode the three candidate classes of a chunk:
 //   plane A | plane B :  route = 1|0,  near-miss = 0|1,  random sentinel = 1|1.
-// PRIOR: also track the weakest near-miss candidate, so that tau = the floor of the k+m old
-// candidates' current scores can warm-start a refresh kernel that wants it (the streaming kernel;
-// the two-sweep kernel derives a tighter bound itself and the third masked pass is a tenth of
-// this kernel's time).
-template <int D, bool PRIOR>
+// The weakest near-miss candidate is tracked as well, so that tau = the floor of the k+m old
+// candidates' current scores can warm-start the refresh.
+template <int D>
 __global__ void __launch_bounds__(NT, 2)
 rescore_dense_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q,
                      const __grid_constant__ CUtensorMap tmap_k, int words, int force_timeout) {
@@ -105,8 +98,7 @@ rescore_dense_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q,
   // A thread reads its ids 16 at a time (16-byte loads where the ledger row allows) and sets
   // their bits with shared-memory reductions (no read-modify-write round trips to wait for).
   // The first two batches are fetched before the pipeline set-up so that their memory round
-  // trip overlaps it.  Without the prior-bound pass (PRIOR = false) the classes are just route
-  // (plane A) and sentinel (plane B): part 0 then skips the random / global slots.
+  // trip overlaps it.
   const int cquarter = warp & 3, cpart = (warp - 2) >> 2;
   const int crow_l = cquarter * 32 + lane;                       // row inside the tile
   const int crow = tm * tcpipe::BM + crow_l;
@@ -115,7 +107,7 @@ rescore_dense_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q,
   // part 0: range 0 = route [0, k), range 1 = sentinel slots [m, sw); part 1: range 0 = [0, sw)
   const int32_t* const ptr0 = cpart == 0 ? p.routes + cg * p.k : p.sentinels + cg * p.sw;
   const int32_t* const ptr1 = p.sentinels + cg * p.sw + p.m;
-  const int n0 = chas ? (cpart == 0 ? p.k : p.sw) : 0, n1 = chas && cpart == 0 && PRIOR ? p.sw - p.m : 0;
+  const int n0 = chas ? (cpart == 0 ? p.k : p.sw) : 0, n1 = chas && cpart == 0 ? p.sw - p.m : 0;
   auto load16 = [&](const int32_t* ptr, int s0, int n, int (&ids)[16]) {
     if (s0 + 16 <= n && (((uintptr_t)(ptr + s0)) & 15u) == 0) {
 #pragma unroll
@@ -174,7 +166,7 @@ rescore_dense_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q,
           if (ok) asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(plane + (uint32_t)(id >> 5) * 4u), "r"(1u << (id & 31)) : "memory");
         }
       };
-      const int cb0 = (part == 0 || !PRIOR) ? 0x7fffffff : p.m;   // range 0: all / the near-miss slots
+      const int cb0 = part == 0 ? 0x7fffffff : p.m;   // range 0: all / the near-miss slots
       or_ids(pre0, 0, cb0);
       or_ids(pre1, pre1_s0, pre1_is1 ? 0x7fffffff : cb0);
       const int n0_max = __reduce_max_sync(FULL, n0), n1_max = __reduce_max_sync(FULL, n1);
@@ -208,7 +200,7 @@ rescore_dense_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q,
       const int wi = t * TPR + part;                       // this thread's word of either plane
       const bool in = alive && wi < words;
       const uint32_t wa = in ? lds(bA + wi * 4u) : 0u, wb = in ? lds(bB + wi * 4u) : 0u;
-      const uint32_t wr = PRIOR ? wa & ~wb : wa, wn = wb & ~wa, ws = wb;
+      const uint32_t wr = wa & ~wb, wn = wb & ~wa, ws = wb;
       const bool work = __any_sync(FULL, (wa | wb) != 0u);
       uint32_t a0[COLS];
       if (work) {
@@ -220,7 +212,7 @@ rescore_dense_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q,
           const float s0 = __uint_as_float(a0[q]);
           min_if(amin, s0, wr, 1u << q);
           max_if(bmax, s0, ws, 1u << q);
-          if constexpr (PRIOR) min_if(nmin, s0, wn, 1u << q);
+          min_if(nmin, s0, wn, 1u << q);
         }
       }
       if (p.debug) {                                         // tests: every candidate's score
@@ -263,7 +255,7 @@ rescore_dense_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q,
         p.flags[g] = flag ? 1 : 0;
         p.alpha[g] = amin;
         p.beta[g] = bmax;
-        p.tau[g] = (PRIOR && p.m > 0) ? fminf(amin, nmin) : ninf;    // floor of the k+m old candidates
+        p.tau[g] = p.m > 0 ? fminf(amin, nmin) : ninf;    // floor of the k+m old candidates
       }
       const int n_flag = __popc(__ballot_sync(FULL, flag));
       const int v_sum = __reduce_add_sync(FULL, flag ? v : 0);
@@ -307,7 +299,7 @@ bool rr_rescore_dense_supported(const RRParams& p) {
 }
 
 cudaError_t rr_launch_rescore_dense(const RRParams& p, const void* qc, const void* kc,
-                                    int force_timeout, bool prior, cudaStream_t st) {
+                                    int force_timeout, cudaStream_t st) {
   int words;
   const size_t smem = smem_need(p, words);
   CUtensorMap tmap, tmap_q;
@@ -317,8 +309,7 @@ cudaError_t rr_launch_rescore_dense(const RRParams& p, const void* qc, const voi
   if (e != cudaSuccess) return e;
   static unsigned long long attr_done = 0;      // devices on which the attributes are set
   e = rr_once_per_device(attr_done, [] {
-    const void* kernels[4] = {(const void*)rescore_dense_kernel<128, true>, (const void*)rescore_dense_kernel<128, false>,
-                              (const void*)rescore_dense_kernel<64, true>, (const void*)rescore_dense_kernel<64, false>};
+    const void* kernels[2] = {(const void*)rescore_dense_kernel<128>, (const void*)rescore_dense_kernel<64>};
     for (const void* k : kernels) {
       const cudaError_t a = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
       if (a != cudaSuccess) return a;
@@ -327,9 +318,7 @@ cudaError_t rr_launch_rescore_dense(const RRParams& p, const void* qc, const voi
     return cudaSuccess;
   });
   if (e != cudaSuccess) return e;
-  auto kernel = p.d == 128 ? (prior ? rescore_dense_kernel<128, true> : rescore_dense_kernel<128, false>)
-                           : (prior ? rescore_dense_kernel<64, true> : rescore_dense_kernel<64, false>);
-  e = rr_launch_pdl(kernel, p.n_tiles, NT, smem, st, p, tmap_q, tmap, words, force_timeout);
+  e = rr_launch_pdl(p.d == 128 ? rescore_dense_kernel<128> : rescore_dense_kernel<64>, p.n_tiles, NT, smem, st, p, tmap_q, tmap, words, force_timeout);
   rr_count_launch();
   return e;
 }
