@@ -175,12 +175,12 @@ class ClockSampler:
 
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the kernels that
 # dominate a high_drift step, from the ncu captures summarised in profiles/
-# (route_sweep_high_drift.md: 199.1 MB anchor / 198.6 MB refresh; rescore_dense_high_drift.md;
-# sentinels_high_drift.md), and the algorithmic bytes per launch of the same launches.  Other
-# workloads report the capture's traffic-to-algorithmic ratio times their own algorithmic bytes
-# and say so.
-NCU_TRAFFIC_BYTES = {"route_fused": ((4 * 199.1e6 + 28 * 198.6e6) / 32, (4 * 203.4e6 + 28 * 196.7e6) / 32),
-                     "rescore_dense": (241.3e6, 203.7e6),
+# (route_rows_high_drift.md, a refresh of 97 % of the rows; rescore_rows_high_drift.md;
+# sentinels_high_drift.md, relay in place only), and the algorithmic bytes per launch of the same
+# launches.  Other workloads report the capture's traffic-to-algorithmic ratio times their own
+# algorithmic bytes and say so.
+NCU_TRAFFIC_BYTES = {"route_fused": (212.0e6, 196.7e6),
+                     "rescore_dense": (238.3e6, 203.7e6),
                      "sentinels": (66.5e6, 0.971 * 262144 * 64 * 4)}
 
 
@@ -599,7 +599,7 @@ def main():
     ap.add_argument("--two-pass", action="store_true",
                     help="route through score rows in scratch + warp-level TopK")
     ap.add_argument("--streaming", action="store_true",
-                    help="route with the streaming fused kernel instead of the two-sweep kernel")
+                    help="route with the streaming kernel instead of the two-sweep kernel")
     ap.add_argument("--inplace", action="store_true",
                     help="relay layers: challenge test inside the routing kernel (one pass over "
                          "the score strip, no compacted second GEMM)")

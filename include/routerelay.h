@@ -76,20 +76,19 @@ typedef struct rr_config {
   int32_t chunk_tokens;    /* >0: also expand routes to token ranges of this chunk size    */
   int32_t debug_outputs;   /* bit 0: relay also stores every candidate score (tests);
                               bit 1: route through the two-pass path (score rows in scratch
-                              + warp-level TopK) even where the fused kernel applies;
+                              + warp-level TopK) even where one kernel does both;
                               bit 2: rescore candidates with the gathered FP32 kernel even
-                              where the tensor-core strip kernel applies;
-                              bit 3 (tests): the two-sweep routing kernel hands every fifth
-                              row to its exact slow path;
-                              bit 4: route with the streaming fused kernel even where the
-                              two-sweep kernel applies;
+                              where a kernel that scores the whole strip applies;
+                              bit 3 (tests): the two-sweep routing kernels hand every fifth
+                              row to their exact slow path;
+                              bit 4: route with the streaming kernel even where a two-sweep
+                              kernel applies;
                               bit 5: relay in place -- the challenge test of Eq. 5 runs inside
                               the routing kernel on the scores of its first sweep (no separate
                               rescoring kernel, no second score GEMM over a compacted list);
                               the results are the same;
-                              bit 8: route with the two-sweep kernel whatever the grid size
-                              (by default grids of less than two waves of CTAs use the
-                              streaming kernel: fewer launches, shorter latency chain);
+                              bit 8: accepted, without effect (the two-sweep kernel is the
+                              default at every grid size);
                               bits 6, 7 (tests): the first wait of the first CTA of the first
                               routing launch (bit 6) / strip rescoring launch (bit 7) of this
                               ledger counts as expired, once: that CTA gives up as after a real
@@ -322,9 +321,10 @@ int rr_bucket_set_status(rr_bucket_set* S, void* stream, uint32_t* status_out);
 /* ---- A minimal consumer of token ranges (Eq. 3) ------------------------------------------------
  * out[i] = softmax(q_i K_R^T * scale) V_R over the tokens R covered by row i's token ranges
  * (views.token_ranges: [rows, slots, 2] = [start, end) per slot, (-1,-1) = empty; per route slot
- * or coalesced).  One warp per row, FP32 arithmetic in ascending token order, so coalesced and
- * per-slot ranges of the same route give bit-identical outputs.  A plain reference consumer, not
- * a tuned attention backend (Section 4.3 leaves the backend unchanged); no token-level mask.
+ * or coalesced).  One CTA per row, FP32 arithmetic; how a row's tokens are split and merged depends
+ * on their numbers in ascending order only, so coalesced and per-slot ranges of the same route give
+ * bit-identical outputs.  A plain reference consumer, not a tuned attention backend (Section 4.3
+ * leaves the backend unchanged); no token-level mask.
  *   ranges  device int32 [rows, slots, 2]       q       device [rows, dh]
  *   keys    device [rows / n_q, tokens, dh]      values  device, same shape as keys
  *   dtype   RR_BF16 or RR_F32 (q, keys, values)  out     device float [rows, dh]
