@@ -52,3 +52,11 @@ def test_best_chunks_in_one_threads_tiles():
         got = led.routes.cpu().numpy()
         assert (got == want).all(axis=1).mean() > 0.999      # (float64 against fp32: near-ties only)
         led.close()
+
+
+@pytest.mark.parametrize("n_q", [1, 32, 33, 65, 97, 128, 129])
+@pytest.mark.parametrize("rho", [0.002, 0.2])
+def test_quarters_without_rows(n_q, rho):
+    """Row tiles whose last quarters (32 rows) are empty, at anchors and on short and long lists."""
+    w = _w(n_q, 300, 64, 12, 8, 6, False).replace(rho=rho)
+    parity.assert_clean(parity.run_teacher_forced(w))
