@@ -914,7 +914,10 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
 // 1024 chunks: 27.1 / 40; keep 48, 576 and 1024 chunks: 57.8 / 80 and 58.9 / 80; with 256 groups,
 // keep 96, 2048 chunks: 119 / 140).  A row that needs more takes the slow path (fewer than 3 in
 // 10^6 at keep 48; a column of 76 entries let 7 in 10^5 through, and the CTA that meets one runs
-// 12 us longer: 289 instead of 265 us on 2048 CTAs).  Beyond 48 the column and the second set of maxima leave room for one CTA per SM.
+// 12 us longer: 289 instead of 265 us on 2048 CTAs).  Beyond 48 the column and the second set of maxima
+// leave room for one CTA per SM, which then waits for its sorts: up to keep 64 (256 groups, 1024 and 2048
+// chunks: 71 / 84 and 72 / 90) a column of 104 entries instead of 152 takes 560 instead of 653 us on 2048
+// CTAs (keep 64, 1024 chunks), 349 instead of 396 us on 1024 (keep 60, 2048 chunks).
 struct Plan { int variant, ring_bytes; size_t smem; };
 
 bool plan(const RRParams& p, Plan& out) {
@@ -923,7 +926,8 @@ bool plan(const RRParams& p, Plan& out) {
   int cap;
   if (keep <= 28) { out.variant = 0; cap = 48; }
   else if (keep <= 48) { out.variant = 1; cap = 80; }
-  else if (keep <= 96) { out.variant = 2; cap = 152; }
+  else if (keep <= 64) { out.variant = 2; cap = 104; }
+  else if (keep <= 96) { out.variant = 3; cap = 152; }
   else return false;
   const int words = (p.n_k + 31) / 32;
   const int stages = p.d == 64 || out.variant != 1 ? 3 : 2;
@@ -936,9 +940,11 @@ bool plan(const RRParams& p, Plan& out) {
 
 typedef void (*Kernel)(RRParams, const __nv_bfloat16*, const CUtensorMap, const int32_t*, uint32_t, int, int, int);
 Kernel kernel_of(int d, int variant) {
-  static const Kernel table[2][3] = {
-      {route_rows_kernel<64, 1, 48, 2, 3, 1>, route_rows_kernel<64, 1, 80, 2, 3, 2>, route_rows_kernel<64, 2, 152, 1, 3, 1>},
-      {route_rows_kernel<128, 1, 48, 2, 3, 1>, route_rows_kernel<128, 1, 80, 2, 2, 2>, route_rows_kernel<128, 2, 152, 1, 3, 1>}};
+  static const Kernel table[2][4] = {
+      {route_rows_kernel<64, 1, 48, 2, 3, 1>, route_rows_kernel<64, 1, 80, 2, 3, 2>, route_rows_kernel<64, 2, 104, 1, 3, 1>,
+       route_rows_kernel<64, 2, 152, 1, 3, 1>},
+      {route_rows_kernel<128, 1, 48, 2, 3, 1>, route_rows_kernel<128, 1, 80, 2, 2, 2>, route_rows_kernel<128, 2, 104, 1, 3, 1>,
+       route_rows_kernel<128, 2, 152, 1, 3, 1>}};
   return table[d == 128 ? 1 : 0][variant];
 }
 
@@ -968,7 +974,7 @@ cudaError_t rr_launch_route_rows(const RRParams& p, const void* qc, const void* 
   static unsigned long long attr_done = 0;      // devices on which the attributes are set
   e = rr_once_per_device(attr_done, [] {
     for (int d = 64; d <= 128; d += 64)
-      for (int v = 0; v < 3; ++v) {
+      for (int v = 0; v < 4; ++v) {
         const cudaError_t a = cudaFuncSetAttribute((const void*)kernel_of(d, v),
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (a != cudaSuccess) return a;
