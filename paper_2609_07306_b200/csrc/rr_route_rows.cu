@@ -910,14 +910,16 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
 
 // ---- configurations ------------------------------------------------------------------------------
 // keep = k + max(m, 1) decides how many entries a row's column needs: the bound lets 1.05-1.25 keep
-// scores pass while keep is at most 3/8 of the groups (mean / largest of 10^5 random rows: keep 24,
-// 1024 chunks: 27.1 / 40; keep 48, 576 and 1024 chunks: 57.8 / 80 and 58.9 / 80; with 256 groups,
-// keep 96, 2048 chunks: 119 / 140).  A row that needs more takes the slow path (fewer than 3 in
-// 10^6 at keep 48; a column of 76 entries let 7 in 10^5 through, and the CTA that meets one runs
-// 12 us longer: 289 instead of 265 us on 2048 CTAs).  Beyond 48 the column and the second set of maxima
-// leave room for one CTA per SM, which then waits for its sorts: up to keep 64 (256 groups, 1024 and 2048
-// chunks: 71 / 84 and 72 / 90) a column of 104 entries instead of 152 takes 560 instead of 653 us on 2048
-// CTAs (keep 64, 1024 chunks), 349 instead of 396 us on 1024 (keep 60, 2048 chunks).
+// scores pass while keep is at most 3/8 of the groups (mean / largest of 2 10^4 to 10^5 random rows;
+// 128 groups, 1024 chunks: keep 24 27 / 40, keep 36 41 / 55, keep 48 59 / 80; 256 groups, 2048 chunks:
+// keep 64 72 / 90, keep 80 94 / 111, keep 96 117 / 142).  A row that needs more takes the slow path, and
+// the CTA that meets one runs 12 us longer (a column of 76 entries at keep 48 let 7 in 10^5 rows
+// through: 289 instead of 265 us on 2048 CTAs).  A longer column than needed lengthens the sorts:
+//   keep 32, 256 x 1024 x 1024: 64 entries 247 us, 80 entries 271 us
+//   keep 64, 256 x 1024 x 1024: 104 entries 560 us, 152 entries 653 us
+//   keep 80, 64 x 2048 x 2048: 128 entries 384 us, 152 entries 406 us
+//   keep 96, 64 x 2048 x 2048: 144 entries 413 us, 152 entries 421 us
+// Beyond 48 the column and the second set of maxima leave room for one CTA per SM.
 struct Plan { int variant, ring_bytes; size_t smem; };
 
 bool plan(const RRParams& p, Plan& out) {
@@ -925,12 +927,14 @@ bool plan(const RRParams& p, Plan& out) {
   if (p.dtype != RR_BF16 || (p.d != 64 && p.d != 128) || p.n_k > RR_MAX_NK) return false;
   int cap;
   if (keep <= 28) { out.variant = 0; cap = 48; }
-  else if (keep <= 48) { out.variant = 1; cap = 80; }
-  else if (keep <= 64) { out.variant = 2; cap = 104; }
-  else if (keep <= 96) { out.variant = 3; cap = 152; }
+  else if (keep <= 36) { out.variant = 1; cap = 64; }
+  else if (keep <= 48) { out.variant = 2; cap = 80; }
+  else if (keep <= 64) { out.variant = 3; cap = 104; }
+  else if (keep <= 80) { out.variant = 4; cap = 128; }
+  else if (keep <= 96) { out.variant = 5; cap = 144; }
   else return false;
   const int words = (p.n_k + 31) / 32;
-  const int stages = p.d == 64 || out.variant != 1 ? 3 : 2;
+  const int stages = p.d == 64 || out.variant != 2 ? 3 : 2;
   int ring = stages * BN * p.d * 2;
   if (ring < words * (int)WORD_PITCH) ring = words * (int)WORD_PITCH;
   out.ring_bytes = (ring + 1023) / 1024 * 1024;
@@ -940,11 +944,11 @@ bool plan(const RRParams& p, Plan& out) {
 
 typedef void (*Kernel)(RRParams, const __nv_bfloat16*, const CUtensorMap, const int32_t*, uint32_t, int, int, int);
 Kernel kernel_of(int d, int variant) {
-  static const Kernel table[2][4] = {
-      {route_rows_kernel<64, 1, 48, 2, 3, 1>, route_rows_kernel<64, 1, 80, 2, 3, 2>, route_rows_kernel<64, 2, 104, 1, 3, 1>,
-       route_rows_kernel<64, 2, 152, 1, 3, 1>},
-      {route_rows_kernel<128, 1, 48, 2, 3, 1>, route_rows_kernel<128, 1, 80, 2, 2, 2>, route_rows_kernel<128, 2, 104, 1, 3, 1>,
-       route_rows_kernel<128, 2, 152, 1, 3, 1>}};
+  static const Kernel table[2][6] = {
+      {route_rows_kernel<64, 1, 48, 2, 3, 1>, route_rows_kernel<64, 1, 64, 2, 3, 2>, route_rows_kernel<64, 1, 80, 2, 3, 2>,
+       route_rows_kernel<64, 2, 104, 1, 3, 1>, route_rows_kernel<64, 2, 128, 1, 3, 1>, route_rows_kernel<64, 2, 144, 1, 3, 1>},
+      {route_rows_kernel<128, 1, 48, 2, 3, 1>, route_rows_kernel<128, 1, 64, 2, 3, 2>, route_rows_kernel<128, 1, 80, 2, 2, 2>,
+       route_rows_kernel<128, 2, 104, 1, 3, 1>, route_rows_kernel<128, 2, 128, 1, 3, 1>, route_rows_kernel<128, 2, 144, 1, 3, 1>}};
   return table[d == 128 ? 1 : 0][variant];
 }
 
@@ -974,7 +978,7 @@ cudaError_t rr_launch_route_rows(const RRParams& p, const void* qc, const void* 
   static unsigned long long attr_done = 0;      // devices on which the attributes are set
   e = rr_once_per_device(attr_done, [] {
     for (int d = 64; d <= 128; d += 64)
-      for (int v = 0; v < 4; ++v) {
+      for (int v = 0; v < 6; ++v) {
         const cudaError_t a = cudaFuncSetAttribute((const void*)kernel_of(d, v),
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (a != cudaSuccess) return a;

@@ -1,5 +1,6 @@
 """The two-threads-per-row routing kernel at the edges of its dispatch and of its tiles: column
-capacities (keep = k + max(m, 1) at 28 | 29, 48 | 49, 64 | 65, 96 | 97), key chunks around the 64-wide tiles
+capacities (keep = k + max(m, 1) at 28 | 29, 36 | 37, 48 | 49, 64 | 65, 80 | 81,
+96 | 97), key chunks around the 64-wide tiles
 and the two-tile round of a row's threads, rows that see fewer chunks than they keep, ragged row
 tiles and widths that rule out 16-byte stores."""
 import numpy as np
@@ -18,7 +19,7 @@ def _w(n_q, n_k, d, k, m, r, causal, **kw):
                            centroids=12, rho=0.2, causal=causal, seed=21, **kw)
 
 
-@pytest.mark.parametrize("k,m", [(20, 8), (20, 9), (32, 16), (33, 16), (47, 0), (16, 32), (32, 32), (33, 32), (64, 32), (65, 32), (3, 1)])
+@pytest.mark.parametrize("k,m", [(20, 8), (20, 9), (24, 12), (24, 13), (32, 16), (33, 16), (47, 0), (16, 32), (32, 32), (33, 32), (48, 32), (49, 32), (64, 32), (65, 32), (3, 1)])
 def test_widths_around_the_column_capacities(k, m):
     rep = parity.run_teacher_forced(_w(150, 700, 128, k, m, 9, True, causal_offset=550))
     parity.assert_clean(rep)
