@@ -15,6 +15,9 @@
 // phases, not the GEMM (which is therefore simply issued twice); everything is laid out so that
 // TWO CTAs fit an SM (113 KB of shared memory, 96 registers, 256 TMEM columns each) and one CTA's
 // latency-bound phases hide behind the other's sweeps.
+// 256 x 1024 x 1024, keep 48: 276 us, where four threads per row with one CTA per SM and a sentinel
+// kernel behind it (rr_route_sweep.cu, rr_sentinels.cu) took 350 + 60; 64 x 2048 x 2048, keep 96: 413 us,
+// where the streaming kernel took 521.  Issue slots are 47 % busy, the tensor pipe 13 %, DRAM 9 %.
 //
 // Sweep 1 (threshold before filtering): scores are cut to bf16 (the upper half of the float, one
 // byte permute per two scores) and each thread keeps packed running maxima of 64 NG groups of

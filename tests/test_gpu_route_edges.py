@@ -1,8 +1,7 @@
 """The two-threads-per-row routing kernel at the edges of its dispatch and of its tiles: column
-capacities (keep = k + max(m, 1) at 28 | 29, 36 | 37, 48 | 49, 64 | 65, 80 | 81,
-96 | 97), key chunks around the 64-wide tiles
-and the two-tile round of a row's threads, rows that see fewer chunks than they keep, ragged row
-tiles and widths that rule out 16-byte stores."""
+capacities (keep = k + max(m, 1) at 28 | 29, 36 | 37, 48 | 49, 64 | 65, 80 | 81, 96 | 97), key chunks
+around the 64-wide tiles and the two-tile round of a row's threads, rows that see fewer chunks than
+they keep, ragged row tiles and widths that rule out 16-byte stores."""
 import numpy as np
 import pytest
 import torch
