@@ -19,6 +19,7 @@
 // A first version (one warp per row, a lane per token for K, two passes) read K with 32 separate
 // cache lines per load and computed every logit twice: 2400 us for 2048 rows of 1024 tokens, dh = 128,
 // bf16; this one: 99 us (1.07 GB of K and V rows, 10.9 TB/s from L2).  Widths that do not split into 16-byte lanes keep it.
+#include <type_traits>
 #include "rr_common.cuh"
 
 namespace {
@@ -151,10 +152,13 @@ attend_row_kernel(const int32_t* __restrict__ ranges, int slots, int n_q, const 
   for (int e = 0; e < E; ++e) acc[e] = 0.f;
   const float ninf = __int_as_float(0xff800000);
   float m = ninf, l = 0.f;
-  for (int b0 = warp * 32; b0 < n_tok; b0 += WARPS * 32) {
+  // One block of 32 tokens, or the row's last one with n_last: its empty places repeat the last token with
+  // weight 0 -- and a value of 0, as its row may hold an infinity.
+  auto block = [&](int b0, int n_last, auto whole) {
+    const int n = decltype(whole)::value ? 32 : n_last;
     // token of number b0 + lane: the last slot that starts at or before it (empty slots start where
     // the next one does and are passed over)
-    const int num = min(b0 + lane, n_tok - 1);
+    const int num = b0 + min(lane, n - 1);
     int s = 0, hi = slots;
     while (hi - s > 1) { const int mid = (s + hi) >> 1; if (s_first[mid] <= num) s = mid; else hi = mid; }
     const int tok = s_base[s] + num;
@@ -179,12 +183,13 @@ attend_row_kernel(const int32_t* __restrict__ ranges, int slots, int n_q, const 
       }
     }
     const int my = sub * TP + grp;                             // this lane's token of the block
-    const float logit = b0 + my < n_tok ? part[0] * scale : ninf;
+    const float logit = my < n ? part[0] * scale : ninf;
     float bm = logit;
 #pragma unroll
     for (int off = 16; off; off >>= 1) bm = fmaxf(bm, __shfl_xor_sync(FULL, bm, off));
-    const float m_new = fmaxf(m, bm), f = expf(m - m_new);     // (exp(-inf) = 0 at the first block)
-    const float w = expf(logit - m_new);
+    // while the warp has met nothing but -inf, 0 stands for the maximum (-inf - -inf would be NaN)
+    const float m_new = fmaxf(m, bm), m_ref = m_new == ninf ? 0.f : m_new;
+    const float f = expf(m - m_ref), w = expf(logit - m_ref);
     l = l * f + w;
     m = m_new;
 #pragma unroll
@@ -195,9 +200,12 @@ attend_row_kernel(const int32_t* __restrict__ ranges, int slots, int n_q, const 
       Lane<T>::load(vp + (size_t)__shfl_sync(FULL, tok, i * TP + grp) * DH, vv);
       const float wi = __shfl_sync(FULL, w, grp * LPT + i);
 #pragma unroll
-      for (int e = 0; e < E; ++e) acc[e] = fmaf(wi, vv[e], acc[e]);
+      for (int e = 0; e < E; ++e) acc[e] = fmaf(wi, i * TP + grp < n ? vv[e] : 0.f, acc[e]);
     }
-  }
+  };
+  int b0 = warp * 32;
+  for (; b0 + 32 <= n_tok; b0 += WARPS * 32) block(b0, 32, std::true_type());
+  if (b0 < n_tok) block(b0, n_tok - b0, std::false_type());
 #pragma unroll
   for (int off = LPT; off < 32; off <<= 1)                     // the token groups of the warp
 #pragma unroll
@@ -216,7 +224,8 @@ attend_row_kernel(const int32_t* __restrict__ ranges, int slots, int n_q, const 
   float fw[WARPS], den = 0.f;
 #pragma unroll
   for (int w = 0; w < WARPS; ++w) { fw[w] = s_m[w] == ninf ? 0.f : expf(s_m[w] - mx); den = fmaf(s_l[w], fw[w], den); }
-  const float inv = den > 0.f ? 1.f / den : 0.f;
+  // (tokens that all score -inf have no softmax: NaN, as without the split; a row without tokens gives 0)
+  const float inv = den > 0.f ? 1.f / den : n_tok > 0 ? __int_as_float(0x7fc00000) : 0.f;
   for (int e = threadIdx.x; e < DH; e += WARPS * 32) {
     float o = 0.f;
 #pragma unroll
