@@ -177,6 +177,13 @@ cudaError_t rr_launch_reset(const RRParams& p, cudaStream_t st);
 
 void rr_count_launch(int n = 1);
 
+// SMs of the current device (148 where the query fails).
+inline int rr_sm_count() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return 148;
+  return sms;
+}
+
 // Function attributes (dynamic shared-memory limit) are per device: `setup` runs the first time
 // the calling site is reached with a given device current, under a lock, and the device is
 // marked done only if it returned cudaSuccess (so a failure is retried, and no other host

@@ -184,7 +184,7 @@ cudaError_t rr_launch_route_f32(const RRParams& p, const void* qc, const void* k
   if (e != cudaSuccess) return e;
   // 16 rows per CTA reuse Kc twice as often; 8 where 16 would not give every SM two CTAs, or would
   // not fit the score rows
-  const int R = p.P * ((p.n_q + 15) / 16) >= 2 * 148 && smem_bytes(p, 16) <= MAX_SMEM ? 16 : 8;
+  const int R = p.P * ((p.n_q + 15) / 16) >= 2 * rr_sm_count() && smem_bytes(p, 16) <= MAX_SMEM ? 16 : 8;
   const int grid = p.P * ((p.n_q + R - 1) / R);
   const cudaError_t l = rr_launch_pdl(kernel_of(p.d, R), grid, NT, smem_bytes(p, R), st, p, (const float*)qc,
                                       (const float*)kc, anchor, (uint32_t)layer);

@@ -460,8 +460,9 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
 
   if (warp == 0) {
     // The Kc tiles beyond the ring are asked into L2, and so are the Qc rows of the CTA that will
-    // start about when this one ends (CTAs start in index order as SMs fall free), so that its
-    // set-up waits for L2 instead of DRAM.  Hints only: nothing depends on them.
+    // start about when this one ends (CTAs start in index order as SMs fall free: the one that comes
+    // cta_stride = CTAs per SM x SMs later), so that its set-up waits for L2 instead of DRAM.  Hints
+    // only: nothing depends on them.
     for (int t = pre + lane; t < n_tiles; t += 32) tma_prefetch_l2_tile(tmap_ptr, t * BN, prob);
     const int nb = (int)blockIdx.x + cta_stride;
     if (nb < (int)gridDim.x) {
@@ -923,7 +924,7 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
 //   keep 80, 64 x 2048 x 2048: 128 entries 384 us, 152 entries 406 us
 //   keep 96, 64 x 2048 x 2048: 144 entries 413 us, 152 entries 421 us
 // Beyond 48 the column and the second set of maxima leave room for one CTA per SM.
-struct Plan { int variant, ring_bytes; size_t smem; };
+struct Plan { int variant, ctas, ring_bytes; size_t smem; };   // ctas: per SM
 
 bool plan(const RRParams& p, Plan& out) {
   const int keep = p.k + (p.m > 0 ? p.m : 1);
@@ -936,6 +937,7 @@ bool plan(const RRParams& p, Plan& out) {
   else if (keep <= 80) { out.variant = 4; cap = 128; }
   else if (keep <= 96) { out.variant = 5; cap = 144; }
   else return false;
+  out.ctas = out.variant <= 2 ? 2 : 1;
   const int words = (p.n_k + 31) / 32;
   const int stages = p.d == 64 || out.variant != 2 ? 3 : 2;
   int ring = stages * BN * p.d * 2;
@@ -991,7 +993,7 @@ cudaError_t rr_launch_route_rows(const RRParams& p, const void* qc, const void* 
   });
   if (e != cudaSuccess) return e;
   e = rr_launch_pdl(kernel_of(p.d, pl.variant), p.n_tiles, NT, pl.smem, st, p, (const __nv_bfloat16*)qc, tmap, row_list,
-                    (uint32_t)layer, hooks, pl.ring_bytes, 2 * 148);
+                    (uint32_t)layer, hooks, pl.ring_bytes, pl.ctas * rr_sm_count());
   rr_count_launch();
   return e;
 }

@@ -990,9 +990,7 @@ cudaError_t rr_launch_route_sweep(const RRParams& p, const void* qc, const void*
                                 227 * 1024);
   });
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 148;                     // CTAs resident at a time: one per SM
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = rr_sm_count();              // CTAs resident at a time: one per SM
   const __nv_bfloat16* q = (const __nv_bfloat16*)qc;
   const size_t smem = smem_bytes(p.d);
   if (p.d == 128)
