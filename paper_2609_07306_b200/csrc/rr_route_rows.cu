@@ -14,7 +14,8 @@
 // What bounds this kernel is the instruction issue of the selection and the latency of its
 // phases, not the GEMM (which is therefore simply issued twice); everything is laid out so that
 // TWO CTAs fit an SM (113 KB of shared memory, 96 registers, 256 TMEM columns each) and one CTA's
-// latency-bound phases hide behind the other's sweeps.
+// latency-bound phases hide behind the other's sweeps, as far as a row's column allows it (see the
+// configurations at the end).
 // 256 x 1024 x 1024, keep 48: 276 us, where four threads per row with one CTA per SM and a sentinel
 // kernel behind it (rr_route_sweep.cu, rr_sentinels.cu) took 350 + 60; 64 x 2048 x 2048, keep 96: 413 us,
 // where the streaming kernel took 521.  Issue slots are 47 % busy, the tensor pipe 13 %, DRAM 9 %.
@@ -174,6 +175,9 @@ __device__ __forceinline__ uint32_t fixed_bits(float s, float tau, float scale) 
   return __float_as_uint(fmaf(t, 8355000.0f, 8388608.0f));
 }
 
+__device__ __forceinline__ void tmem_ld_cols(uint32_t a, uint32_t (&r)[32]) { tmem_ld_32x32(a, r); }
+__device__ __forceinline__ void tmem_ld_cols(uint32_t a, uint32_t (&r)[16]) { tmem_ld_32x16(a, r); }
+
 // ---- threshold filter of sweep 2 ------------------------------------------------------------
 // One score: if it passes, {score, chunk id} goes to [w] and w moves on by one entry (a compare,
 // an id add and three predicated instructions; EDGE: ids >= v never pass, one compare more).  Two
@@ -274,6 +278,7 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   constexpr int TILE = BN * D * 2;
   static_assert(STAGES >= 2 && STAGES <= ACC_STAGES, "see produce()");
   constexpr int M = CAP / 2;                               // entries per half column
+  constexpr int S1 = NG == 2 && CTAS == 2 ? 16 : SLICE;    // columns per load of sweep 1 (64 maxima and 96 registers: no room for 32 scores)
   extern __shared__ __align__(1024) uint8_t smem_raw[];    // (checked below: the swizzle needs it)
   uint8_t* smem = smem_raw;
   uint8_t* sB = smem;                                      // Kc ring; after the sweeps: keys, bitmap
@@ -512,24 +517,24 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
           const int t = t0 + TPR * c;
           if (t < n_tiles && tile_wait(t)) {
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const int col0 = t * BN + h * SLICE;
-              uint32_t acc[SLICE];
-              if (col0 < vmaxw) tmem_ld_32x32(acc_addr(t, h), acc);
-              if (h == 1) tile_release(t);
-              if (col0 + SLICE <= vminw) {
+            for (int h = 0; h < BN / S1; ++h) {
+              const int col0 = t * BN + h * S1;
+              uint32_t acc[S1];
+              if (col0 < vmaxw) tmem_ld_cols(acc_lane + (uint32_t)((t % ACC_STAGES) * BN + h * S1), acc);
+              if (h == BN / S1 - 1) tile_release(t);
+              if (col0 + S1 <= vminw) {
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
+                for (int i = 0; i < S1 / 2; ++i) {
                   const uint32_t pk = __byte_perm(acc[2 * i], acc[2 * i + 1], 0x7632);   // upper halves: bf16, cut
-                  asm("max.bf16x2 %0, %0, %1;" : "+r"(mx[c * 32 + h * 16 + i]) : "r"(pk));
+                  asm("max.bf16x2 %0, %0, %1;" : "+r"(mx[c * 32 + h * (S1 / 2) + i]) : "r"(pk));
                 }
               } else if (col0 < vmaxw) {                     // some row's last chunk lies inside
                 const int nv = v - col0;
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
+                for (int i = 0; i < S1 / 2; ++i) {
                   const uint32_t pk = __byte_perm(acc[2 * i], acc[2 * i + 1], 0x7632);
                   const uint32_t pm = 2 * i + 1 < nv ? pk : (pk & 0xffffu) | 0xff800000u;
-                  asm("max.bf16x2 %0, %0, %1;" : "+r"(mx[c * 32 + h * 16 + i]) : "r"(2 * i < nv ? pm : 0xff80ff80u));
+                  asm("max.bf16x2 %0, %0, %1;" : "+r"(mx[c * 32 + h * (S1 / 2) + i]) : "r"(2 * i < nv ? pm : 0xff80ff80u));
                 }
               }
             }
@@ -564,11 +569,12 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
         const float la = A(max(a - 1, 0)), lb = B(max(b - 1, 0));
         return fminf(a > 0 ? la : pinf, b > 0 ? lb : pinf);
       };
-      // shares in proportion to the threads' non-empty groups
+      // shares in proportion to the threads' non-empty groups (64 NG at most), of which a thread has
+      // kept the g0 / g1 largest maxima
       const int q = v / BN, rem = v % BN;
-      const int g0 = min(64, ((q + 1) / 2) * BN + ((q & 1) == 0 ? rem : 0));
-      const int g1 = min(64, (q / 2) * BN + ((q & 1) == 1 ? rem : 0));
-      int share0 = g1 == 0 ? T : g1 == 64 ? (T + 1) / 2 : (int)((float)(T * g0) / (float)(g0 + g1) + 0.5f);
+      const int c0 = min(64 * NG, ((q + 1) / 2) * BN + ((q & 1) == 0 ? rem : 0)), g0 = min(64, c0);
+      const int c1 = min(64 * NG, (q / 2) * BN + ((q & 1) == 1 ? rem : 0)), g1 = min(64, c1);
+      int share0 = c1 == 0 ? T : c1 == 64 * NG ? (T + 1) / 2 : (int)((float)(T * c0) / (float)(c0 + c1) + 0.5f);
       share0 = min(g0, max(share0, T - g1));
       int share = j == 0 ? share0 : T - share0;
       float bound = share_bound(share);
@@ -771,8 +777,8 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
       if (width > 0) {
         if (width <= 16) gather_ids<16>(col, e0, m0, e1, m1, bits, sampling, dst, width, vec, go);
         else if (width <= 32) gather_ids<32>(col, e0, m0, e1, m1, bits, sampling, dst, width, vec, go);
-        else if (NG == 1 || width <= 64) gather_ids<64>(col, e0, m0, e1, m1, bits, sampling, dst, width, vec, go);
-        else if constexpr (NG > 1) gather_ids<128>(col, e0, m0, e1, m1, bits, sampling, dst, width, vec, go);
+        else if (NG == 1 || CTAS == 2 || width <= 64) gather_ids<64>(col, e0, m0, e1, m1, bits, sampling, dst, width, vec, go);
+        else if constexpr (NG > 1 && CTAS == 1) gather_ids<128>(col, e0, m0, e1, m1, bits, sampling, dst, width, vec, go);
       }
     }
     PH_LAP(6);
@@ -913,47 +919,70 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
 }
 
 // ---- configurations ------------------------------------------------------------------------------
-// keep = k + max(m, 1) decides how many entries a row's column needs: the bound lets 1.05-1.25 keep
-// scores pass while keep is at most 3/8 of the groups (mean / largest of 2 10^4 to 10^5 random rows;
-// 128 groups, 1024 chunks: keep 24 27 / 40, keep 36 41 / 55, keep 48 59 / 80; 256 groups, 2048 chunks:
-// keep 64 72 / 90, keep 80 94 / 111, keep 96 117 / 142).  A row that needs more takes the slow path, and
-// the CTA that meets one runs 12 us longer (a column of 76 entries at keep 48 let 7 in 10^5 rows
-// through: 289 instead of 265 us on 2048 CTAs).  A longer column than needed lengthens the sorts:
-//   keep 32, 256 x 1024 x 1024: 64 entries 247 us, 80 entries 271 us
-//   keep 64, 256 x 1024 x 1024: 104 entries 560 us, 152 entries 653 us
-//   keep 80, 64 x 2048 x 2048: 128 entries 384 us, 152 entries 406 us
-//   keep 96, 64 x 2048 x 2048: 144 entries 413 us, 152 entries 421 us
-// Beyond 48 the column and the second set of maxima leave room for one CTA per SM.
+// keep = k + max(m, 1) and the number of key chunks decide how many entries a row's column needs: with
+// 64 groups to a thread and class the bound lets 1.05-1.25 keep scores pass (few where a group holds
+// one chunk or two).  A row that needs more takes the slow path, and the CTA that meets one runs 12 us
+// longer (a column of 76 entries at keep 48 let 7 in 10^5 rows of 1024 chunks through: 289 instead of
+// 265 us on 2048 CTAs); a longer column than needed lengthens the sorts (keep 32, 256 x 1024 x 1024:
+// 64 entries 247 us, 80 entries 271 us; keep 80, 64 x 2048 x 2048: 128 entries 384, 152 entries 406).
+// What counts most is whether two CTAs fit an SM: 80 entries are the longest column that lets them.
+//   keep <= 48: 128 groups (mean / largest of 10^5 random rows of 1024 chunks: keep 24 27 / 40, keep 36
+//               41 / 55, keep 48 59 / 80);
+//   beyond:     256 groups, whose maxima alone are 64 registers of a thread: sweep 1 then takes 16 scores
+//               at a time where two CTAs leave it 96 registers.
+// MOST: most kept chunks for a column of 80, 88, 104 or 128 entries, by the number of key chunks.  The
+// lines lie where fewer than 1 row in 10^4 needs more, over random and clustered rows of every length up
+// to n_k (largest of 99.98 % of them: keep 70 of 256 chunks 77, keep 62 of 512 77, keep 58 of 1024 76,
+// keep 56 of 2048 75); rows of 161 to 200 chunks (three and a bit tiles) are the worst of their length.
+// 9 layers at rho = 0.2, two CTAs of 80 or 88 entries against one of 104 or 128 entries:
+//   256 x 256 x 256, keep 65: 1189 and 1874 us; 200 x 140 x 1024, keep 58: 959 and 1059; 64 x 2048 x 2048,
+//   keep 56: 2495 and 3171; 128 x 512 x 512 (d 64), keep 68: 1140 and 1679.
+// Past a line the slow path costs more than the second CTA gives: 40 x 500 x 450, keep 66 at rho = 0.004 514
+// us with one CTA, 636 with two; 100 x 300 x 2048 (d 64), keep 60: 887 and 1380.  Shorter columns where one
+// CTA runs: 128 x 512 x 512, keep 80 of 104 entries instead of 128 1631 and 1754 us; 200 x 140 x 1024, keep 88
+// of 128 instead of 144 entries, past the line of 84: 1829 and 1633.
 struct Plan { int variant, ctas, ring_bytes; size_t smem; };   // ctas: per SM
+constexpr int WIDE = 3;              // variants from here on: 256 groups
+constexpr int cap_of(int variant, int d) {
+  constexpr int caps[7] = {48, 64, 80, 80, 104, 128, 144};
+  return variant == WIDE && d == 64 ? 88 : caps[variant];      // (smaller Kc tiles leave room for 8 entries more)
+}
+constexpr struct { int n_k, cap80, cap88, cap104, cap128; } MOST[] = {
+    {256, 70, 76, 80, 84}, {320, 66, 72, 80, 84}, {512, 62, 68, 76, 84}, {1024, 58, 64, 70, 84},
+    {1536, 56, 62, 64, 80}, {2048, 56, 0, 64, 80}, {RR_MAX_NK, 0, 0, 64, 80}};   // (0: the bitmaps leave no room for two)
 
 bool plan(const RRParams& p, Plan& out) {
   const int keep = p.k + (p.m > 0 ? p.m : 1);
-  if (p.dtype != RR_BF16 || (p.d != 64 && p.d != 128) || p.n_k > RR_MAX_NK) return false;
-  int cap;
-  if (keep <= 28) { out.variant = 0; cap = 48; }
-  else if (keep <= 36) { out.variant = 1; cap = 64; }
-  else if (keep <= 48) { out.variant = 2; cap = 80; }
-  else if (keep <= 64) { out.variant = 3; cap = 104; }
-  else if (keep <= 80) { out.variant = 4; cap = 128; }
-  else if (keep <= 96) { out.variant = 5; cap = 144; }
-  else return false;
-  out.ctas = out.variant <= 2 ? 2 : 1;
+  if (p.dtype != RR_BF16 || (p.d != 64 && p.d != 128) || p.n_k > RR_MAX_NK || keep > 96) return false;
+  if (keep <= 48) {
+    out.variant = keep <= 28 ? 0 : keep <= 36 ? 1 : 2;
+  } else {
+    int i = 0;
+    while (p.n_k > MOST[i].n_k) ++i;
+    const auto& most = MOST[i];
+    // (two CTAs leave a thread 96 registers, in which it orders 64 ids at most)
+    out.variant = keep <= (p.d == 64 ? most.cap88 : most.cap80) && p.k <= 64 && p.m <= 64 ? WIDE
+                  : keep <= most.cap104 ? 4 : keep <= most.cap128 ? 5 : 6;
+  }
   const int words = (p.n_k + 31) / 32;
-  const int stages = p.d == 64 || out.variant != 2 ? 3 : 2;
+  const int stages = p.d == 64 || (out.variant != 2 && out.variant != WIDE) ? 3 : 2;
   int ring = stages * BN * p.d * 2;
   if (ring < words * (int)WORD_PITCH) ring = words * (int)WORD_PITCH;
   out.ring_bytes = (ring + 1023) / 1024 * 1024;
-  out.smem = (size_t)out.ring_bytes + CTL_BYTES + (size_t)cap * SLOT_PITCH;
+  out.smem = (size_t)out.ring_bytes + CTL_BYTES + (size_t)cap_of(out.variant, p.d) * SLOT_PITCH;
+  out.ctas = out.variant <= WIDE && 2 * (out.smem + 1024) <= 228 * 1024 ? 2 : 1;
   return out.smem <= 227 * 1024;
 }
 
 typedef void (*Kernel)(RRParams, const __nv_bfloat16*, const CUtensorMap, const int32_t*, uint32_t, int, int, int);
 Kernel kernel_of(int d, int variant) {
-  static const Kernel table[2][6] = {
+  static const Kernel table[2][7] = {
       {route_rows_kernel<64, 1, 48, 2, 3, 1>, route_rows_kernel<64, 1, 64, 2, 3, 2>, route_rows_kernel<64, 1, 80, 2, 3, 2>,
-       route_rows_kernel<64, 2, 104, 1, 3, 1>, route_rows_kernel<64, 2, 128, 1, 3, 1>, route_rows_kernel<64, 2, 144, 1, 3, 1>},
+       route_rows_kernel<64, 2, 88, 2, 3, 2>, route_rows_kernel<64, 2, 104, 1, 3, 1>, route_rows_kernel<64, 2, 128, 1, 3, 1>,
+       route_rows_kernel<64, 2, 144, 1, 3, 1>},
       {route_rows_kernel<128, 1, 48, 2, 3, 1>, route_rows_kernel<128, 1, 64, 2, 3, 2>, route_rows_kernel<128, 1, 80, 2, 2, 2>,
-       route_rows_kernel<128, 2, 104, 1, 3, 1>, route_rows_kernel<128, 2, 128, 1, 3, 1>, route_rows_kernel<128, 2, 144, 1, 3, 1>}};
+       route_rows_kernel<128, 2, 80, 2, 2, 2>, route_rows_kernel<128, 2, 104, 1, 3, 1>, route_rows_kernel<128, 2, 128, 1, 3, 1>,
+       route_rows_kernel<128, 2, 144, 1, 3, 1>}};
   return table[d == 128 ? 1 : 0][variant];
 }
 
@@ -983,7 +1012,7 @@ cudaError_t rr_launch_route_rows(const RRParams& p, const void* qc, const void* 
   static unsigned long long attr_done = 0;      // devices on which the attributes are set
   e = rr_once_per_device(attr_done, [] {
     for (int d = 64; d <= 128; d += 64)
-      for (int v = 0; v < 6; ++v) {
+      for (int v = 0; v < 7; ++v) {
         const cudaError_t a = cudaFuncSetAttribute((const void*)kernel_of(d, v),
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (a != cudaSuccess) return a;

@@ -1,5 +1,5 @@
 """The two-threads-per-row routing kernel at the edges of its dispatch and of its tiles: column
-capacities (keep = k + max(m, 1) at 28 | 29, 36 | 37, 48 | 49, 64 | 65, 80 | 81, 96 | 97), key chunks
+capacities (keep = k + max(m, 1) at 28 | 29, 36 | 37, 48 | 49, 96 | 97, and by the number of key chunks), key chunks
 around the 64-wide tiles and the two-tile round of a row's threads, rows that see fewer chunks than
 they keep, ragged row tiles and widths that rule out 16-byte stores."""
 import numpy as np
@@ -60,3 +60,39 @@ def test_quarters_without_rows(n_q, rho):
     """Row tiles whose last quarters (32 rows) are empty, at anchors and on short and long lists."""
     w = _w(n_q, 300, 64, 12, 8, 6, False).replace(rho=rho)
     parity.assert_clean(parity.run_teacher_forced(w))
+
+
+# most kept chunks of the two-CTA columns and of the columns after them, by key chunks and head width, and
+# the first that needs the next column
+@pytest.mark.parametrize("n_k,d,keep", [
+    (256, 128, 70), (256, 128, 71), (257, 128, 67), (320, 128, 66), (512, 128, 62), (513, 128, 62), (1024, 128, 58),
+    (1025, 128, 57), (2048, 128, 56), (2049, 128, 56), (190, 128, 70), (256, 64, 76), (256, 64, 77), (320, 64, 72),
+    (512, 64, 68), (1024, 64, 64), (1536, 64, 62), (1537, 64, 60), (320, 64, 80), (512, 128, 77), (1024, 64, 85)])
+@pytest.mark.parametrize("causal", [False, True])
+def test_columns_by_key_chunks(n_k, d, keep, causal):
+    w = _w(131, n_k, d, keep - 24, 24, 9, causal, causal_offset=max(0, n_k - 131) if causal else 0)
+    parity.assert_clean(parity.run_teacher_forced(w))
+
+
+@pytest.mark.parametrize("k,m", [(64, 1), (65, 1), (1, 64), (1, 65), (45, 9)])
+def test_wide_routes_of_unequal_parts(k, m):
+    """Ids ordered per thread: up to 64 where two CTAs share an SM, more beyond."""
+    parity.assert_clean(parity.run_teacher_forced(_w(140, 250, 64, k, m, 4, False)))
+
+
+@pytest.mark.parametrize("n_k,d", [(256, 128), (200, 64)])
+def test_slow_path_of_wide_routes(n_k, d):
+    """Every fifth row through the exact slow path, then rows whose scores all tie (every row)."""
+    w = _w(140, n_k, d, 40, 16, 8, True)
+    parity.assert_clean(parity.run_teacher_forced(w, force_slow_rows=True))
+    led = RouteLedger(config_from_workload(w))
+    led.route_anchor(torch.zeros(2, 140, d, device="cuda", dtype=torch.bfloat16),
+                     torch.zeros(2, n_k, d, device="cuda", dtype=torch.bfloat16), 0)
+    torch.cuda.synchronize()
+    r = led.routes.cpu().numpy().reshape(2, 140, 40)
+    s = led.sentinels.cpu().numpy().reshape(2, 140, -1)[:, :, :16]
+    for i in range(140):
+        kk, nn = min(40, i + 1), min(16, max(0, i + 1 - 40))
+        assert (np.sort(r[:, i, :kk], 1) == np.arange(kk)).all() and (r[:, i, kk:] == -1).all(), i
+        assert (np.sort(s[:, i, :nn], 1) == np.arange(kk, kk + nn)).all() and (s[:, i, nn:] == -1).all(), i
+    led.close()
