@@ -599,7 +599,7 @@ def main():
     ap.add_argument("--two-pass", action="store_true",
                     help="route through score rows in scratch + warp-level TopK")
     ap.add_argument("--streaming", action="store_true",
-                    help="route with the streaming kernel instead of the two-sweep kernel")
+                    help="route with the streaming kernel instead of the default one")
     ap.add_argument("--inplace", action="store_true",
                     help="relay layers: challenge test inside the routing kernel (one pass over "
                          "the score strip, no compacted second GEMM)")

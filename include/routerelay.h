@@ -81,14 +81,14 @@ typedef struct rr_config {
                               where a kernel that scores the whole strip applies;
                               bit 3 (tests): the two-sweep routing kernels hand every fifth
                               row to their exact slow path;
-                              bit 4: route with the streaming kernel even where a two-sweep
+                              bit 4: route with the streaming kernel even where the two-sweep
                               kernel applies;
-                              bit 5: relay in place -- the challenge test of Eq. 5 runs inside
-                              the routing kernel on the scores of its first sweep (no separate
-                              rescoring kernel, no second score GEMM over a compacted list);
-                              the results are the same;
-                              bit 8: accepted, without effect (the two-sweep kernel is the
-                              default at every grid size);
+                              bit 5: relay in place -- where k + max(m, 1) <= 48 and n_k <= 1024
+                              (without bits 1 and 4) a kernel of its own routes, and where also
+                              k + m + r + g <= 64 the challenge test of Eq. 5 runs inside it on the
+                              scores of its first sweep (no separate rescoring kernel, no second
+                              score GEMM over a compacted list); the results are the same;
+                              bit 8: accepted, without effect;
                               bits 6, 7 (tests): the first wait of the first CTA of the first
                               routing launch (bit 6) / strip rescoring launch (bit 7) of this
                               ledger counts as expired, once: that CTA gives up as after a real

@@ -49,9 +49,9 @@ def test_sweep_shapes(n, two_pass, gathered):
 @pytest.mark.parametrize("wl", ["moderate", "sweep512", "sweep1024"])
 def test_routing_kernel_variants(wl, variant):
     """The other ways a bf16 row can be routed in one kernel (and "inplace": the relay whose
-    challenge test runs inside the routing kernel, Section 3.2 and 4.2 in one pass): the two-sweep kernel with every
-    fifth row handed to its exact slow path (complete score row in shared memory + warp-level
-    radix select), and the streaming kernel that serves the shapes the two-sweep kernel does
+    challenge test runs inside a routing kernel, Section 3.2 and 4.2 in one pass): the two-sweep kernels with every
+    fifth row handed to their exact slow path (complete score row in shared memory + warp-level
+    radix select), and the streaming kernel that serves the shapes the default kernel does
     not hold."""
     w = {"moderate": W.moderate(),
          "sweep512": W.sweep(512, 0.15).replace(heads=4, layers=4, anchor_every=3),
@@ -62,14 +62,19 @@ def test_routing_kernel_variants(wl, variant):
     parity.assert_clean(rep)
 
 
-@pytest.mark.parametrize("two_sweep", [True, False])
-def test_degenerate_all_equal_scores_bf16(two_sweep):
-    """All-zero bf16 inputs through the fused routing kernels (every score ties; in the two-sweep
-    kernel every list is one run of equal keys, so all rows take its slow path; a grid this small
-    uses the streaming kernel unless the two-sweep kernel is asked for): TopK must take the
-    smallest ids under the causal mask, margin 0."""
+def test_in_place_request_beyond_its_candidates():
+    """k + m + r above what the test in place holds: its kernel routes from the refresh list instead."""
+    w = W.sweep(512, 0.15).replace(heads=2, r=20, layers=4, anchor_every=3)
+    parity.assert_clean(parity.run_teacher_forced(w, inplace=True))
+
+
+@pytest.mark.parametrize("streaming", [False, True], ids=["default", "streaming"])
+def test_degenerate_all_equal_scores_bf16(streaming):
+    """All-zero bf16 inputs through the fused routing kernels (every score ties; in the default
+    kernel every column overflows, so all rows take its slow path; the streaming kernel meets one bin
+    that holds the whole row): TopK must take the smallest ids under the causal mask, margin 0."""
     w = W.moderate().replace(heads=2)
-    led = RouteLedger(config_from_workload(w, two_sweep=two_sweep))
+    led = RouteLedger(config_from_workload(w, streaming=streaming))
     z = torch.zeros(1, w.problems, w.n_q, w.d, device="cuda", dtype=torch.bfloat16)
     led.route_anchor(z, z, 0)
     torch.cuda.synchronize()
@@ -309,9 +314,9 @@ def test_token_ranges(two_pass, coalesce):
     led.close()
 
 
-@pytest.mark.parametrize("two_sweep", [False, True], ids=["streaming", "two_sweep"])
+@pytest.mark.parametrize("streaming", [True, False], ids=["streaming", "default"])
 @pytest.mark.parametrize("wl", ["moderate", "sweep_1024_rho0.30_4heads"])
-def test_free_running_summary_matches_oracle(wl, two_sweep):
+def test_free_running_summary_matches_oracle(wl, streaming):
     """All layers without teacher forcing: recall / refreshed-row / score-pair fractions of
     the device run agree with the oracle's run up to the ambiguous rows.  Second case: the
     routing-scale sweep at 1024 chunks and the highest drift (4 of its 32 heads, 16 layers)."""
@@ -320,7 +325,7 @@ def test_free_running_summary_matches_oracle(wl, two_sweep):
     p = parity.oracle_params(w)
     res, summ = O.run_layers(W.as_float32(q).astype(np.float64), W.as_float32(k).astype(np.float64),
                              p, w.anchor_every)
-    led = RouteLedger(config_from_workload(w, two_sweep=two_sweep))
+    led = RouteLedger(config_from_workload(w, streaming=streaming))
     hit = tot = 0
     for l in range(w.layers):
         fn = led.route_anchor if w.is_anchor(l) else led.route_relay
