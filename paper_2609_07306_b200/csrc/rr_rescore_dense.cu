@@ -29,25 +29,9 @@ constexpr int NCONS = tcpipe::BM * TPR, NT = 64 + NCONS;
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr uint32_t PITCH = tcpipe::BM * 4;          // debug score column: one word per row
 
-__device__ __forceinline__ uint32_t lds(uint32_t a) {
-  uint32_t v; asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(a) : "memory"); return v;
-}
-__device__ __forceinline__ void sts(uint32_t a, uint32_t v) {
-  asm volatile("st.shared.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
 __device__ __forceinline__ void consumers_sync() {            // the NCONS consumer threads only
   asm volatile("bar.sync 1, %0;" ::"n"(NCONS) : "memory");
 }
-// acc = min(acc, s) / max(acc, s) if (word & bit): a predicate and a predicated instruction
-__device__ __forceinline__ void min_if(float& acc, float s, uint32_t word, uint32_t bit) {
-  asm("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tand.b32 t, %2, %3;\n\tsetp.ne.u32 p, t, 0;\n\t"
-      "@p min.f32 %0, %0, %1;\n\t}" : "+f"(acc) : "f"(s), "r"(word), "r"(bit));
-}
-__device__ __forceinline__ void max_if(float& acc, float s, uint32_t word, uint32_t bit) {
-  asm("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tand.b32 t, %2, %3;\n\tsetp.ne.u32 p, t, 0;\n\t"
-      "@p max.f32 %0, %0, %1;\n\t}" : "+f"(acc) : "f"(s), "r"(word), "r"(bit));
-}
-
 #ifdef RR_PHASE_TIMING
 // cycles per phase, kept in registers and added to the global totals once per warp
 __device__ unsigned long long g_rd_phase[8];
@@ -151,7 +135,7 @@ rescore_dense_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q,
     // ---- ledger row -> this thread's plane of the row's bitmap -----------------------------
     {
       const uint32_t plane = part == 0 ? bA : bB;
-      for (int w = 0; w < words; ++w) sts(plane + w * 4u, 0u);
+      for (int w = 0; w < words; ++w) sts32(plane + w * 4u, 0u);
       RD_LAP(4);
       int n_ok = 0; bool bad = false;
       // candidates are charged once: part 0 counts what it sets, part 1 only the near-miss slots
@@ -199,7 +183,7 @@ rescore_dense_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q,
       static_assert(COLS == 32, "a thread's share of a tile is one bitmap word");
       const int wi = t * TPR + part;                       // this thread's word of either plane
       const bool in = alive && wi < words;
-      const uint32_t wa = in ? lds(bA + wi * 4u) : 0u, wb = in ? lds(bB + wi * 4u) : 0u;
+      const uint32_t wa = in ? lds32(bA + wi * 4u) : 0u, wb = in ? lds32(bB + wi * 4u) : 0u;
       const uint32_t wr = wa & ~wb, wn = wb & ~wa, ws = wb;
       const bool work = __any_sync(FULL, (wa | wb) != 0u);
       uint32_t a0[COLS];
@@ -218,7 +202,7 @@ rescore_dense_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q,
       if (p.debug) {                                         // tests: every candidate's score
         if (work) {
 #pragma unroll
-          for (int q = 0; q < COLS; ++q) sts(col + (sh + q) * PITCH, a0[q]);
+          for (int q = 0; q < COLS; ++q) sts32(col + (sh + q) * PITCH, a0[q]);
         }
         consumers_sync();
         if (alive && part == 0 && row >= 0) {
@@ -228,7 +212,7 @@ rescore_dense_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q,
             const int id = s < p.k ? route[s] : sent[s - p.k];
             const int rel = id - t * BN;
             if (id >= 0 && id < v && rel >= 0 && rel < BN)
-              p.cand_scores[(size_t)g * p.c + s] = __uint_as_float(lds(col + (uint32_t)rel * PITCH));
+              p.cand_scores[(size_t)g * p.c + s] = __uint_as_float(lds32(col + (uint32_t)rel * PITCH));
           }
         }
         consumers_sync();
@@ -240,15 +224,15 @@ rescore_dense_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q,
     RD_FLUSH();
     // ---- the second thread of each row hands its partial results to the first ---------------
     if (part != 0) {
-      sts(xch_base + r * 4u, __float_as_uint(amin));
-      sts(xch_base + PITCH + r * 4u, __float_as_uint(bmax));
-      sts(xch_base + 2u * PITCH + r * 4u, __float_as_uint(nmin));
+      sts32(xch_base + r * 4u, __float_as_uint(amin));
+      sts32(xch_base + PITCH + r * 4u, __float_as_uint(bmax));
+      sts32(xch_base + 2u * PITCH + r * 4u, __float_as_uint(nmin));
     }
     consumers_sync();
     if (part == 0) {
-      amin = fminf(amin, __uint_as_float(lds(xch_base + r * 4u)));
-      bmax = fmaxf(bmax, __uint_as_float(lds(xch_base + PITCH + r * 4u)));
-      nmin = fminf(nmin, __uint_as_float(lds(xch_base + 2u * PITCH + r * 4u)));
+      amin = fminf(amin, __uint_as_float(lds32(xch_base + r * 4u)));
+      bmax = fmaxf(bmax, __uint_as_float(lds32(xch_base + PITCH + r * 4u)));
+      nmin = fminf(nmin, __uint_as_float(lds32(xch_base + 2u * PITCH + r * 4u)));
       const bool ok = alive && row >= 0;
       const bool flag = ok && rr_challenge(p, g, amin, bmax);
       if (ok) {

@@ -49,22 +49,6 @@ static_assert(sizeof(Ctl) <= CTL_BYTES, "control block too large");
 __device__ __forceinline__ void consumers_sync() {   // the consumer warps only
   asm volatile("bar.sync 1, %0;" ::"n"(CONS_WARPS * 32) : "memory");
 }
-__device__ __forceinline__ uint32_t lds32(uint32_t a) {
-  uint32_t v; asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(a) : "memory"); return v;
-}
-__device__ __forceinline__ void sts32(uint32_t a, uint32_t v) {
-  asm volatile("st.shared.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-// acc = min(acc, s) / max(acc, s) if (word & bit)
-__device__ __forceinline__ void min_if(float& acc, float s, uint32_t word, uint32_t bit) {
-  asm("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tand.b32 t, %2, %3;\n\tsetp.ne.u32 p, t, 0;\n\t"
-      "@p min.f32 %0, %0, %1;\n\t}" : "+f"(acc) : "f"(s), "r"(word), "r"(bit));
-}
-__device__ __forceinline__ void max_if(float& acc, float s, uint32_t word, uint32_t bit) {
-  asm("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tand.b32 t, %2, %3;\n\tsetp.ne.u32 p, t, 0;\n\t"
-      "@p max.f32 %0, %0, %1;\n\t}" : "+f"(acc) : "f"(s), "r"(word), "r"(bit));
-}
-
 template <int D>
 __global__ void __launch_bounds__(NT, 2)
 rescore_rows_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,

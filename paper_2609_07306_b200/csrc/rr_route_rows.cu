@@ -45,6 +45,7 @@
 // memory, and a warp per row runs the radix select of the two-pass path.  Every mbarrier wait is
 // bounded.
 #include "rr_common.cuh"
+#include "rr_networks.cuh"
 #include "rr_sm100.cuh"
 #include "rr_warp_topk.cuh"
 
@@ -75,29 +76,12 @@ constexpr int CTL_BYTES = 1024;
 constexpr int MAIL = 20;                // slot of a half column through which its thread gets the other's messages
 static_assert(sizeof(Ctl) <= CTL_BYTES, "control block too large");
 
-__device__ __forceinline__ uint32_t lds32(uint32_t a) {
-  uint32_t v; asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(a) : "memory"); return v;
-}
-__device__ __forceinline__ float ldsf(uint32_t a) { return __uint_as_float(lds32(a)); }
-__device__ __forceinline__ void lds64(uint32_t a, uint32_t& x, uint32_t& y) {
-  asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(x), "=r"(y) : "r"(a) : "memory");
-}
-__device__ __forceinline__ void sts32(uint32_t a, uint32_t v) {
-  asm volatile("st.shared.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-__device__ __forceinline__ void sts64(uint32_t a, uint32_t x, uint32_t y) {
-  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
-}
 // the two warps that share a quarter of the rows (64 threads), barrier ids 1..4
 __device__ __forceinline__ void quarter_sync(int quarter) {
   asm volatile("bar.sync %0, 64;" ::"r"(quarter + 1) : "memory");
 }
 
-// ---- packed compare-exchange networks ---------------------------------------------------------
-// Batcher's odd-even merge sort as a compile-time network (descending): every index is a
-// template constant, so the array stays in registers.  N a power of two; LIMIT < N prunes the
-// network to its first LIMIT inputs (inputs from LIMIT on would hold the smallest key and sit
-// last, and a compare-exchange with such an input changes nothing).
+// ---- packed compare-exchanges -----------------------------------------------------------------
 struct DescBF2 {                     // two bf16 lists at a time
   static __device__ __forceinline__ void ce(uint32_t& a, uint32_t& b) {
     uint32_t hi, lo;
@@ -121,30 +105,6 @@ struct AscU2 {                       // two lists of 16-bit values at a time
   static __device__ __forceinline__ void ce(uint32_t& a, uint32_t& b) {
     const uint32_t hi = __vmaxu2(a, b), lo = __vminu2(a, b);
     a = lo; b = hi;
-  }
-};
-template <int LO, int N, int R, class OP, int LIMIT> struct OEMerge {
-  static __device__ __forceinline__ void run(uint32_t* x) {
-    constexpr int M = R * 2;
-    if constexpr (M < N) {
-      OEMerge<LO, N, M, OP, LIMIT>::run(x);
-      OEMerge<LO + R, N, M, OP, LIMIT>::run(x);
-#pragma unroll
-      for (int i = LO + R; i + R < LO + N; i += M)
-        if (i + R < LIMIT) OP::ce(x[i], x[i + R]);
-    } else {
-      if constexpr (LO + R < LIMIT) OP::ce(x[LO], x[LO + R]);
-    }
-  }
-};
-template <int LO, int N, class OP, int LIMIT> struct OESort {
-  static __device__ __forceinline__ void run(uint32_t* x) {
-    if constexpr (N > 1 && LO < LIMIT) {
-      constexpr int M = N / 2;
-      OESort<LO, M, OP, LIMIT>::run(x);
-      OESort<LO + M, M, OP, LIMIT>::run(x);
-      OEMerge<LO, N, 1, OP, LIMIT>::run(x);
-    }
   }
 };
 __host__ __device__ constexpr int pow2_at_least(int n) { int p = 1; while (p < n) p *= 2; return p; }

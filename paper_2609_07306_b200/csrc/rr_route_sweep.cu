@@ -42,6 +42,7 @@
 // complete score rows in shared memory, and a warp per row runs the radix select of the
 // two-pass path on them.  Every mbarrier wait is bounded.
 #include "rr_common.cuh"
+#include "rr_networks.cuh"
 #include "rr_sm100.cuh"
 #include "rr_warp_topk.cuh"
 
@@ -92,57 +93,10 @@ constexpr int BUF_BYTES = CAPJ * ENTRY_PITCH;             // 128 KB
 static_assert(HARD_SLOTS * MAX_NK * 4 + SEL_WARPS * (256 + BM_WORDS) * 4 <= BUF_BYTES,
               "slow-path rows and per-warp scratch must fit the list area");
 
-__device__ __forceinline__ uint32_t lds32(uint32_t a) {
-  uint32_t v; asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(a) : "memory"); return v;
-}
-__device__ __forceinline__ void sts32(uint32_t a, uint32_t v) {
-  asm volatile("st.shared.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-__device__ __forceinline__ void lds64(uint32_t a, uint32_t& x, uint32_t& y) {
-  asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(x), "=r"(y) : "r"(a) : "memory");
-}
-__device__ __forceinline__ void sts64(uint32_t a, uint32_t x, uint32_t y) {
-  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
-}
 // the four warps that share a quarter of the rows (128 threads), barrier ids 1..4
 __device__ __forceinline__ void quarter_sync(int quarter) {
   asm volatile("bar.sync %0, 128;" ::"r"(quarter + 1) : "memory");
 }
-
-// Batcher's odd-even merge sort as a compile-time network (descending): every index is a
-// template constant, so the array stays in registers.  N a power of two.
-template <class T> struct DescF {
-  static __device__ __forceinline__ void ce(T& a, T& b) { const T hi = fmaxf(a, b), lo = fminf(a, b); a = hi; b = lo; }
-};
-template <class T> struct DescU {
-  static __device__ __forceinline__ void ce(T& a, T& b) { const T hi = max(a, b), lo = min(a, b); a = hi; b = lo; }
-};
-// LIMIT < N prunes the network to its first LIMIT inputs: valid when the inputs from LIMIT on hold
-// the smallest key and sit last, since a compare-exchange with such an input changes nothing.
-template <int LO, int N, int R, class T, class OP, int LIMIT> struct OEMerge {
-  static __device__ __forceinline__ void run(T* x) {
-    constexpr int M = R * 2;
-    if constexpr (M < N) {
-      OEMerge<LO, N, M, T, OP, LIMIT>::run(x);
-      OEMerge<LO + R, N, M, T, OP, LIMIT>::run(x);
-#pragma unroll
-      for (int i = LO + R; i + R < LO + N; i += M)
-        if (i + R < LIMIT) OP::ce(x[i], x[i + R]);
-    } else {
-      if constexpr (LO + R < LIMIT) OP::ce(x[LO], x[LO + R]);
-    }
-  }
-};
-template <int LO, int N, class T, class OP, int LIMIT = LO + N> struct OESort {
-  static __device__ __forceinline__ void run(T* x) {
-    if constexpr (N > 1 && LO < LIMIT) {
-      constexpr int M = N / 2;
-      OESort<LO, M, T, OP, LIMIT>::run(x);
-      OESort<LO + M, M, T, OP, LIMIT>::run(x);
-      OEMerge<LO, N, 1, T, OP, LIMIT>::run(x);
-    }
-  }
-};
 
 // ---- sorting one list of sweep 2 ------------------------------------------------------------
 // The list (n <= LIMIT <= 32 entries {score, id} at base + e * ENTRY_PITCH, in ascending chunk id)
@@ -163,7 +117,7 @@ __device__ __forceinline__ bool sort_list(uint32_t base, int n) {
       key[e] = e < n ? ((ok & ~31u) | (uint32_t)(31 - e)) : 0u;
     }
   }
-  OESort<0, CAPJ, uint32_t, DescU<uint32_t>, LIMIT>::run(key);
+  OESort<0, CAPJ, DescU, LIMIT>::run(key);
   bool same = false, run3 = false;
 #pragma unroll
   for (int i = 0; i + 1 < LIMIT; ++i) same |= key[i + 1] >= 32u && ((key[i] ^ key[i + 1]) < 32u);
@@ -657,7 +611,7 @@ route_sweep_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
       asm volatile("bar.sync 5, %0;" ::"n"(SEL_WARPS * 32) : "memory");
     }
     PH_LAP(0);
-    OESort<0, SLICE, float, DescF<float>, SLICE>::run(mx);
+    OESort<0, SLICE, DescF, SLICE>::run(mx);
     // The row's keep-th largest group maximum (over the 128 groups of its four threads) has keep
     // distinct scores of the row at or above it: a valid inclusive lower bound of the row's
     // keep-th largest score, and the tightest one the maxima give (about 1.2 keep scores pass;
