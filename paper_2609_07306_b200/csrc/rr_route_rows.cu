@@ -885,12 +885,13 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
 // longer (a column of 76 entries at keep 48 let 7 in 10^5 rows of 1024 chunks through: 289 instead of
 // 265 us on 2048 CTAs); a longer column than needed lengthens the sorts (keep 32, 256 x 1024 x 1024:
 // 64 entries 247 us, 80 entries 271 us; keep 80, 64 x 2048 x 2048: 128 entries 384, 152 entries 406).
-// What counts most is whether two CTAs fit an SM: 80 entries are the longest column that lets them.
+// What counts most is whether two CTAs fit an SM: 80 entries are the longest column that lets them
+// (88 at d = 64).
 //   keep <= 48: 128 groups (mean / largest of 10^5 random rows of 1024 chunks: keep 24 27 / 40, keep 36
 //               41 / 55, keep 48 59 / 80);
 //   beyond:     256 groups, whose maxima alone are 64 registers of a thread: sweep 1 then takes 16 scores
 //               at a time where two CTAs leave it 96 registers.
-// MOST: most kept chunks for a column of 80, 88, 104 or 128 entries, by the number of key chunks.  The
+// MOST: most kept chunks for a column of 80, 88 (d = 64), 104 or 128 entries, by the number of key chunks.  The
 // lines lie where fewer than 1 row in 10^4 needs more, over random and clustered rows of every length up
 // to n_k (largest of 99.98 % of them: keep 70 of 256 chunks 77, keep 62 of 512 77, keep 58 of 1024 76,
 // keep 56 of 2048 75); rows of 161 to 200 chunks (three and a bit tiles) are the worst of their length.
@@ -902,11 +903,7 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
 // CTA runs: 128 x 512 x 512, keep 80 of 104 entries instead of 128 1631 and 1754 us; 200 x 140 x 1024, keep 88
 // of 128 instead of 144 entries, past the line of 84: 1829 and 1633.
 struct Plan { int variant, ctas, ring_bytes; size_t smem; };   // ctas: per SM
-constexpr int WIDE = 3;              // variants from here on: 256 groups
-constexpr int cap_of(int variant, int d) {
-  constexpr int caps[7] = {48, 64, 80, 80, 104, 128, 144};
-  return variant == WIDE && d == 64 ? 88 : caps[variant];      // (smaller Kc tiles leave room for 8 entries more)
-}
+constexpr int VARIANTS = 8, CAPS[VARIANTS] = {48, 64, 80, 80, 88, 104, 128, 144};
 constexpr struct { int n_k, cap80, cap88, cap104, cap128; } MOST[] = {
     {256, 70, 76, 80, 84}, {320, 66, 72, 80, 84}, {512, 62, 68, 76, 84}, {1024, 58, 64, 70, 84},
     {1536, 56, 62, 64, 80}, {2048, 56, 0, 64, 80}, {RR_MAX_NK, 0, 0, 64, 80}};   // (0: the bitmaps leave no room for two)
@@ -920,29 +917,32 @@ bool plan(const RRParams& p, Plan& out) {
     int i = 0;
     while (p.n_k > MOST[i].n_k) ++i;
     const auto& most = MOST[i];
-    // (two CTAs leave a thread 96 registers, in which it orders 64 ids at most)
-    out.variant = keep <= (p.d == 64 ? most.cap88 : most.cap80) && p.k <= 64 && p.m <= 64 ? WIDE
-                  : keep <= most.cap104 ? 4 : keep <= most.cap128 ? 5 : 6;
+    const bool narrow = p.k <= 64 && p.m <= 64;      // (with 96 registers a thread orders 64 ids at most)
+    // 88 entries fit twice at d = 64 only, where the Kc tiles are smaller; they spill a few registers and
+    // gain nothing where every CTA has an SM to itself (3 x 489 x 489, keep 53: 88 entries 531 us, 104
+    // entries with one CTA per SM 525, 80 entries 518)
+    out.variant = narrow && keep <= most.cap80 ? 3 : narrow && p.d == 64 && keep <= most.cap88 && p.n_tiles > rr_sm_count() ? 4
+                  : keep <= most.cap104 ? 5 : keep <= most.cap128 ? 6 : 7;
   }
   const int words = (p.n_k + 31) / 32;
-  const int stages = p.d == 64 || (out.variant != 2 && out.variant != WIDE) ? 3 : 2;
+  const int stages = p.d == 64 || (out.variant != 2 && out.variant != 3) ? 3 : 2;
   int ring = stages * BN * p.d * 2;
   if (ring < words * (int)WORD_PITCH) ring = words * (int)WORD_PITCH;
   out.ring_bytes = (ring + 1023) / 1024 * 1024;
-  out.smem = (size_t)out.ring_bytes + CTL_BYTES + (size_t)cap_of(out.variant, p.d) * SLOT_PITCH;
-  out.ctas = out.variant <= WIDE && 2 * (out.smem + 1024) <= 228 * 1024 ? 2 : 1;
+  out.smem = (size_t)out.ring_bytes + CTL_BYTES + (size_t)CAPS[out.variant] * SLOT_PITCH;
+  out.ctas = out.variant <= 4 && 2 * (out.smem + 1024) <= 228 * 1024 ? 2 : 1;
   return out.smem <= 227 * 1024;
 }
 
 typedef void (*Kernel)(RRParams, const __nv_bfloat16*, const CUtensorMap, const int32_t*, uint32_t, int, int, int);
 Kernel kernel_of(int d, int variant) {
-  static const Kernel table[2][7] = {
+  static const Kernel table[2][VARIANTS] = {
       {route_rows_kernel<64, 1, 48, 2, 3, 1>, route_rows_kernel<64, 1, 64, 2, 3, 2>, route_rows_kernel<64, 1, 80, 2, 3, 2>,
-       route_rows_kernel<64, 2, 88, 2, 3, 2>, route_rows_kernel<64, 2, 104, 1, 3, 1>, route_rows_kernel<64, 2, 128, 1, 3, 1>,
-       route_rows_kernel<64, 2, 144, 1, 3, 1>},
+       route_rows_kernel<64, 2, 80, 2, 3, 2>, route_rows_kernel<64, 2, 88, 2, 3, 2>, route_rows_kernel<64, 2, 104, 1, 3, 1>,
+       route_rows_kernel<64, 2, 128, 1, 3, 1>, route_rows_kernel<64, 2, 144, 1, 3, 1>},
       {route_rows_kernel<128, 1, 48, 2, 3, 1>, route_rows_kernel<128, 1, 64, 2, 3, 2>, route_rows_kernel<128, 1, 80, 2, 2, 2>,
-       route_rows_kernel<128, 2, 80, 2, 2, 2>, route_rows_kernel<128, 2, 104, 1, 3, 1>, route_rows_kernel<128, 2, 128, 1, 3, 1>,
-       route_rows_kernel<128, 2, 144, 1, 3, 1>}};
+       route_rows_kernel<128, 2, 80, 2, 2, 2>, nullptr, route_rows_kernel<128, 2, 104, 1, 3, 1>,
+       route_rows_kernel<128, 2, 128, 1, 3, 1>, route_rows_kernel<128, 2, 144, 1, 3, 1>}};
   return table[d == 128 ? 1 : 0][variant];
 }
 
@@ -972,7 +972,8 @@ cudaError_t rr_launch_route_rows(const RRParams& p, const void* qc, const void* 
   static unsigned long long attr_done = 0;      // devices on which the attributes are set
   e = rr_once_per_device(attr_done, [] {
     for (int d = 64; d <= 128; d += 64)
-      for (int v = 0; v < 7; ++v) {
+      for (int v = 0; v < VARIANTS; ++v) {
+        if (!kernel_of(d, v)) continue;
         const cudaError_t a = cudaFuncSetAttribute((const void*)kernel_of(d, v),
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (a != cudaSuccess) return a;

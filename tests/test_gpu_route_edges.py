@@ -74,6 +74,13 @@ def test_columns_by_key_chunks(n_k, d, keep, causal):
     parity.assert_clean(parity.run_teacher_forced(w))
 
 
+@pytest.mark.parametrize("n_k,keep", [(256, 71), (256, 76), (256, 77), (320, 72), (512, 68), (1024, 64), (1536, 62)])
+def test_columns_of_grids_beyond_the_sms(n_k, keep):
+    """The column that needs more CTAs than SMs to pay (d = 64): 160 problems, three of them checked."""
+    w = _w(70, n_k, 64, keep - 20, 20, 7, True, causal_offset=n_k - 70).replace(heads=160, layers=2)
+    parity.assert_clean(parity.run_teacher_forced(w, check_problems=[0, 77, 159]))
+
+
 @pytest.mark.parametrize("k,m", [(64, 1), (65, 1), (1, 64), (1, 65), (45, 9)])
 def test_wide_routes_of_unequal_parts(k, m):
     """Ids ordered per thread: up to 64 where two CTAs share an SM, more beyond."""
