@@ -118,10 +118,17 @@ __device__ __forceinline__ bool rr_challenge(const RRParams& p, int g, float alp
 // ---- programmatic dependent launch ---------------------------------------------------------
 // A layer is a chain of short kernels.  Launched with rr_launch_pdl, a kernel may start while its
 // predecessor in the stream drains: it sets itself up and calls rr_pdl_wait() before it reads
-// anything an earlier kernel writes (inputs included: they may come from the caller's kernels).
-// rr_pdl_trigger() lets the successor start; every kernel calls it AFTER its own wait, so that
-// whatever ran before a kernel has finished by the time the kernel after it starts.  Both are no-ops
-// in a kernel launched the ordinary way.  Every path through such a kernel waits.
+// anything its predecessor writes.  rr_pdl_trigger() lets the successor start.  Both are no-ops in a
+// kernel launched the ordinary way.  What makes it safe:
+//   1. A kernel that triggers after its own wait starts its successor only when everything before
+//      itself has finished (the caller's copies and kernels, whose results are the inputs, included).
+//   2. Every path through a kernel waits before it ends, so a kernel's end means that all before it
+//      has ended, and a wait for the predecessor is a wait for everything before.
+//   3. All kernels but one trigger after their wait.  The one is the routing kernel at an anchor: its
+//      predecessor is the anchor's fill, which by 1 has let it start when the inputs were complete and
+//      all earlier layers were done, and which writes nothing that it reads or writes.  It triggers and
+//      works without waiting for the fill and waits before it ends (by 2 its successor, which waits
+//      for it before anything else, finds both done).
 __device__ __forceinline__ void rr_pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void rr_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <class... P, class... A>

@@ -15,7 +15,9 @@
 // Scoring the whole strip costs n_k / c times the multiply-adds of the candidates alone, but reuses
 // every Kc row R times; the gathered form (rr_rescore.cu) moves c Kc rows per query row and needs a
 // second GEMM and a second kernel for the refresh (10 x 384 x 192, c = 48: 135 + 7 + 9 us a relay layer,
-// this kernel 21).  It is bound by the FP32 pipe and by the select's latency.
+// this kernel 21).  At that size (480 CTAs of 8 rows) it is bound by latency, not by the FP32 pipe, which
+// needs 1.3 us: Kc loads with nothing loaded ahead, warps without a chunk at the barrier, and where
+// rows are routed the select's shared-memory round trips (two thirds of an anchor's instructions).
 #include "rr_warp_topk.cuh"
 
 namespace {

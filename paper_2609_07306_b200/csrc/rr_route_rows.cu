@@ -267,8 +267,9 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
     rr_pdl_wait();
     return;
   }
-  // The predecessor writes the refresh list; at an anchor it only fills in book-keeping, and the
-  // inputs have been complete since it started (see rr_launch_pdl).
+  // The predecessor writes the refresh list; at an anchor it is the fill, which only writes
+  // book-keeping that is not read here, and has triggered after its own wait: the inputs are complete.
+  // The wait for it is then at the end of every path (see rr_pdl_wait).
   if (row_list_arg) rr_pdl_wait();
   // a relay call that the forced-anchor policy turned into full routing has the identity list:
   // take the anchor's path (consecutive rows, no gathers through the list)
