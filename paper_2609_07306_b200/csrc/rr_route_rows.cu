@@ -901,12 +901,12 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
 //   keep 56: 2495 and 3171; 128 x 512 x 512 (d 64), keep 68: 1140 and 1679.
 // Past a line the slow path costs more than the second CTA gives: 40 x 500 x 450, keep 66 at rho = 0.004 514
 // us with one CTA, 636 with two; 100 x 300 x 2048 (d 64), keep 60: 887 and 1380.  Shorter columns where one
-// CTA runs: 128 x 512 x 512, keep 80 of 104 entries instead of 128 1631 and 1754 us; 200 x 140 x 1024, keep 88
-// of 128 instead of 144 entries, past the line of 84: 1829 and 1633.
+// CTA runs: 256 x 256 x 256, keep 80 of 104 entries instead of 128 1793 and 1889 us, keep 88 of 128 instead of
+// 144 1950 and 2043; 200 x 140 x 1024, keep 88 of 128 instead of 144 entries, past the line of 84: 1829 and 1633.
 struct Plan { int variant, ctas, ring_bytes; size_t smem; };   // ctas: per SM
 constexpr int VARIANTS = 8, CAPS[VARIANTS] = {48, 64, 80, 80, 88, 104, 128, 144};
 constexpr struct { int n_k, cap80, cap88, cap104, cap128; } MOST[] = {
-    {256, 70, 76, 80, 84}, {320, 66, 72, 80, 84}, {512, 62, 68, 76, 84}, {1024, 58, 64, 70, 84},
+    {256, 70, 76, 80, 92}, {320, 66, 72, 80, 84}, {512, 62, 68, 76, 84}, {1024, 58, 64, 70, 84},
     {1536, 56, 62, 64, 80}, {2048, 56, 0, 64, 80}, {RR_MAX_NK, 0, 0, 64, 80}};   // (0: the bitmaps leave no room for two)
 
 bool plan(const RRParams& p, Plan& out) {

@@ -67,7 +67,7 @@ def test_quarters_without_rows(n_q, rho):
 @pytest.mark.parametrize("n_k,d,keep", [
     (256, 128, 70), (256, 128, 71), (257, 128, 67), (320, 128, 66), (512, 128, 62), (513, 128, 62), (1024, 128, 58),
     (1025, 128, 57), (2048, 128, 56), (2049, 128, 56), (190, 128, 70), (256, 64, 76), (256, 64, 77), (320, 64, 72),
-    (512, 64, 68), (1024, 64, 64), (1536, 64, 62), (1537, 64, 60), (320, 64, 80), (512, 128, 77), (1024, 64, 85)])
+    (512, 64, 68), (1024, 64, 64), (1536, 64, 62), (1537, 64, 60), (256, 128, 92), (256, 64, 93), (320, 64, 80), (512, 128, 77), (1024, 64, 85)])
 @pytest.mark.parametrize("causal", [False, True])
 def test_columns_by_key_chunks(n_k, d, keep, causal):
     w = _w(131, n_k, d, keep - 24, 24, 9, causal, causal_offset=max(0, n_k - 131) if causal else 0)
