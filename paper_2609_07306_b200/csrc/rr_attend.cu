@@ -18,7 +18,7 @@
 //   V: the same loads; a lane accumulates the 8 output dimensions it loads.
 // A first version (one warp per row, a lane per token for K, two passes) read K with 32 separate
 // cache lines per load and computed every logit twice: 2400 us for 2048 rows of 1024 tokens, dh = 128,
-// bf16; this one: 99 us (1.07 GB of K and V rows, 10.9 TB/s from L2).  Widths that do not split into 16-byte lanes keep it.
+// bf16; this one: 101 us (1.07 GB of K and V rows, 10.6 TB/s from L2).  Widths that do not split into 16-byte lanes keep it.
 #include <type_traits>
 #include "rr_common.cuh"
 
