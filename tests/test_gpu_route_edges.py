@@ -2,6 +2,8 @@
 capacities (keep = k + max(m, 1) at 28 | 29, 36 | 37, 48 | 49, 96 | 97, and by the number of key chunks), key chunks
 around the 64-wide tiles and the two-tile round of a row's threads, rows that see fewer chunks than
 they keep, ragged row tiles and widths that rule out 16-byte stores."""
+import random
+
 import numpy as np
 import pytest
 import torch
@@ -103,3 +105,42 @@ def test_slow_path_of_wide_routes(n_k, d):
         assert (np.sort(r[:, i, :kk], 1) == np.arange(kk)).all() and (r[:, i, kk:] == -1).all(), i
         assert (np.sort(s[:, i, :nn], 1) == np.arange(kk, kk + nn)).all() and (s[:, i, nn:] == -1).all(), i
     led.close()
+
+
+@pytest.mark.parametrize("kind", ["normal", "ties", "one_threads_tiles", "duplicates", "large", "uneven"])
+def test_wide_columns_equal_the_two_pass_path(kind):
+    """Bit for bit, over random shapes of 49 to 96 kept chunks and scores that strain the bound: the exact
+    select of the two-pass path runs on the same scores (same tile MMAs)."""
+    rng = random.Random(kind)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    for _ in range(8):
+        d, n_q = rng.choice([64, 128]), rng.choice([1, 40, 131, 300])
+        n_k = rng.choice([rng.randint(100, 330), rng.randint(100, 2100)])
+        P = 170 if n_q == 40 and n_k < 600 else 2                          # (more CTAs than SMs)
+        keep = rng.randint(49, 96)
+        m = rng.choice([0, 1, 20, keep // 2, keep - 1])
+        causal = rng.random() < 0.5
+        w = _w(n_q, n_k, d, keep - max(m, 1), m, rng.choice([0, 5, 8]), causal, causal_offset=n_k // 2 if causal else 0,
+               global_sentinels=rng.choice([0, 3])).replace(heads=P)
+        q, k = (torch.randn((P, n, d), generator=g, device="cuda") for n in (n_q, n_k))
+        if kind == "ties":
+            q.round_(); k.round_()
+        elif kind == "one_threads_tiles":
+            k[:, (torch.arange(n_k, device="cuda") // 64) % 2 == 0] += 0.8 * q.mean((0, 1))
+        elif kind == "duplicates":
+            k = k[:, torch.randint(0, n_k // 3, (n_k,), generator=g, device="cuda")]
+        elif kind == "large":
+            q *= 1e18; k *= 1e18
+        elif kind == "uneven":
+            k *= torch.rand((P, n_k, 1), generator=g, device="cuda") ** 4
+        q, k = q.bfloat16().contiguous(), k.bfloat16().contiguous()
+        got = []
+        for two_pass in (False, True):
+            led = RouteLedger(config_from_workload(w, two_pass=two_pass))
+            led.route_anchor(q, k, 3)
+            led.route_relay(q, k, 4)
+            assert led.status() == 0
+            got.append([led.routes.sort(1).values, led.sentinels[:, :m].sort(1).values, led.sentinels[:, m:].clone(),
+                        led.kth_score.clone(), led.margin.clone()])
+            led.close()
+        assert all(torch.equal(a, b) for a, b in zip(*got)), (w, [torch.equal(a, b) for a, b in zip(*got)])
