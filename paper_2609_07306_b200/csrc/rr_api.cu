@@ -81,9 +81,9 @@ RRParams shape_params(const rr_config* cfg) {
   return p;
 }
 
-// Which kernel routes rows.  Two threads per row with two CTAs per SM (rr_route_rows.cu) wherever
-// its shape limits hold; the relay in place (debug bit 5) exists in the four-threads-per-row kernel
-// only; the streaming kernel takes wider routes (and debug bit 4), the two-pass path the rest.
+// Which kernel routes rows.  Two threads per row (up to 28 kept chunks) or four, two CTAs per SM where the column
+// allows it, wherever their shape limits hold; the relay in place on any grid (debug bit 5) exists in the
+// sweep kernel only; the streaming kernel takes wider routes (and debug bit 4), the two-pass path the rest.
 // fp32 inputs are scored, tested and routed in one kernel per row tile, unless the two-pass or the
 // gathered form is asked for (10 problems of 384 x 192, c = 48: relay 135 + 7 + 9 us for gathered test,
 // GEMM and selection).
@@ -96,7 +96,8 @@ bool uses_sweep(const rr_config* cfg) {
 }
 
 bool uses_rows(const rr_config* cfg) {
-  return !(cfg->debug_outputs & (2 | 16)) && !uses_sweep(cfg) && rr_route_rows_supported(shape_params(cfg));
+  const RRParams p = shape_params(cfg);
+  return !(cfg->debug_outputs & (2 | 16)) && !uses_sweep(cfg) && (rr_route_rows_supported(p) || rr_route_quad_supported(p));
 }
 
 bool uses_fused(const rr_config* cfg) {
@@ -178,6 +179,8 @@ int route_layer(rr_ledger* L, const void* qc, const void* kc, int layer, bool an
     LAUNCH(RR_KIND_ANCHOR_FILL, rr_launch_anchor_fill(p, L->dense_pairs_per_layer, st));
     if (L->f32) {
       LAUNCH(RR_KIND_ROUTE_FUSED, rr_launch_route_f32(p, qc, kc, 1, layer, st));
+    } else if (L->quad) {
+      LAUNCH(RR_KIND_ROUTE_FUSED, rr_launch_route_quad(p, qc, kc, nullptr, false, layer, sweep_hooks(L), st));
     } else if (L->rows) {
       LAUNCH(RR_KIND_ROUTE_FUSED, rr_launch_route_rows(p, qc, kc, nullptr, layer, sweep_hooks(L), st));
     } else if (L->sweep) {
@@ -205,6 +208,15 @@ int route_layer(rr_ledger* L, const void* qc, const void* kc, int layer, bool an
       if (p.chunk_tokens > 0) LAUNCH(RR_KIND_EXPAND, rr_launch_expand(p, 0, st));
       return RR_OK;
     }
+    if (L->tests) {
+      // The routing kernel tests every row on the scores of its first sweep; the list is built afterwards.
+      int hooks = sweep_hooks(L);
+      if (L->timeout_shots & 2) { hooks |= 2; L->timeout_shots &= ~2; }
+      LAUNCH(RR_KIND_ROUTE_FUSED, rr_launch_route_quad(p, qc, kc, nullptr, true, layer, hooks, st));
+      LAUNCH(RR_KIND_COMPACT, rr_launch_compact(p, L->dense_pairs_per_layer, st));
+      if (p.chunk_tokens > 0) LAUNCH(RR_KIND_EXPAND, rr_launch_expand(p, 0, st));
+      return RR_OK;
+    }
     if (L->f32) {
       LAUNCH(RR_KIND_ROUTE_FUSED, rr_launch_route_f32(p, qc, kc, 0, layer, st));
       LAUNCH(RR_KIND_COMPACT, rr_launch_compact(p, L->dense_pairs_per_layer, st));
@@ -220,7 +232,9 @@ int route_layer(rr_ledger* L, const void* qc, const void* kc, int layer, bool an
     }
     else LAUNCH(RR_KIND_RESCORE, rr_launch_rescore(p, qc, kc, st));
     LAUNCH(RR_KIND_COMPACT, rr_launch_compact(p, L->dense_pairs_per_layer, st));
-    if (L->rows) {
+    if (L->quad) {
+      LAUNCH(RR_KIND_ROUTE_FUSED, rr_launch_route_quad(p, qc, kc, p.refresh_rows, false, layer, sweep_hooks(L), st));
+    } else if (L->rows) {
       LAUNCH(RR_KIND_ROUTE_FUSED, rr_launch_route_rows(p, qc, kc, p.refresh_rows, layer, sweep_hooks(L), st));
     } else if (L->sweep) {
       LAUNCH(RR_KIND_ROUTE_FUSED, rr_launch_route_sweep(p, qc, kc, p.refresh_rows, layer, 0,
@@ -314,6 +328,7 @@ int rr_ledger_init(const rr_config* cfg, void* dev_ledger, size_t ledger_bytes,
   p.S = (float*)(sb + lay.S);
   L->f32 = uses_f32(cfg);
   L->rows = uses_rows(cfg);
+  L->quad = L->rows && !rr_route_rows_supported(p);
   L->sweep = uses_sweep(cfg);
   L->inplace = L->sweep && (cfg->debug_outputs & 32) && rr_route_sweep_inplace_supported(p);
   L->fused = uses_fused(cfg);
@@ -322,6 +337,7 @@ int rr_ledger_init(const rr_config* cfg, void* dev_ledger, size_t ledger_bytes,
   const bool strip = !(cfg->debug_outputs & 4);
   L->rows_rescore = strip && !L->fused && rr_rescore_rows_supported(p);
   L->dense_rescore = strip && L->fused && rr_rescore_dense_supported(p);
+  L->tests = L->rows && L->rows_rescore && rr_route_quad_tests(p);
   *out = L;
   return RR_OK;
 }

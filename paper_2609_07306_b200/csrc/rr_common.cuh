@@ -48,7 +48,9 @@ struct rr_ledger {
   unsigned call_index;                     // layer calls since reset (parity of the force_state slots)
   int timeout_shots;                       // test hook: forced time-outs still to be fired (bit 0
                                            // routing kernel, bit 1 strip rescoring kernel)
-  bool rows;                               // full routing runs in the two-threads-per-row kernel
+  bool rows;                               // full routing runs in the kernels with two CTAs per SM: two threads per
+  bool quad;                               // row, or four (wider routes)
+  bool tests;                              // relay: challenge test inside the routing kernel with four threads per row
   bool sweep;                              // ... else in the four-threads-per-row kernel
   bool inplace;                            // relay: challenge test inside the routing kernel
   bool fused;                              // ... else in the streaming fused kernel
@@ -157,6 +159,10 @@ cudaError_t rr_launch_route_fused(const RRParams& p, const void* qc, const void*
 bool rr_route_rows_supported(const RRParams& p);
 cudaError_t rr_launch_route_rows(const RRParams& p, const void* qc, const void* kc, const int32_t* row_list,
                                  int layer, int hooks, cudaStream_t st);   // hooks: as below
+bool rr_route_quad_supported(const RRParams& p);
+bool rr_route_quad_tests(const RRParams& p);             // a relay's test is better done by the routing kernel
+cudaError_t rr_launch_route_quad(const RRParams& p, const void* qc, const void* kc, const int32_t* row_list, bool test,
+                                 int layer, int hooks, cudaStream_t st);      // test: relay in place, no list
 bool rr_route_sweep_supported(const RRParams& p);
 cudaError_t rr_launch_route_sweep(const RRParams& p, const void* qc, const void* kc,
                                   const int32_t* row_list, int layer, int inplace, int hooks,

@@ -25,6 +25,7 @@
 // (99 us: more instructions) were no better.
 #include "rr_common.cuh"
 #include "rr_sm100.cuh"
+#include "rr_test_marks.cuh"
 
 using namespace sm100;
 
@@ -164,53 +165,10 @@ rescore_rows_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q, cons
     const float pinf = __int_as_float(0x7f800000);
     const int v = has ? rr_valid_count(row, p.n_k, p.causal, p.causal_offset) : 0;
     // ---- the quarter's ledger rows -> this warp's bitmap (j = 0: routes, 1: sentinels) ---------------
-    int n_cand = 0; bool bad = false;
-    {
-      const int w = j == 0 ? p.k : p.sw;
-      const int row0 = tm * BM + quarter * 32, n_rows = max(0, min(32, p.n_q - row0));
-      const int32_t* const ids = (j == 0 ? p.routes : p.sentinels) + ((size_t)prob * p.n_q + row0) * w;
-      const uint32_t plane = maps_q + (j == 0 ? 0u : (uint32_t)words * 4u);
-      auto mark = [&](int id, int vr, uint32_t map) {
-        bad |= id >= vr;
-        // a shared-memory reduction: marks do not wait for one another
-        asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 a, b;\n\tsetp.lt.u32 p, %1, %2;\n\t"
-                     "shr.u32 a, %1, 5;\n\tmad.lo.u32 a, a, 4, %3;\n\tshf.l.wrap.b32 b, 0, 1, %1;\n\t"
-                     "@p red.shared.or.b32 [a], b;\n\t@p add.s32 %0, %0, 1;\n\t}"
-                     : "+r"(n_cand) : "r"(id), "r"(vr), "r"(map) : "memory");
-      };
-      const bool vec = (w & 3) == 0;
-      const int per = vec ? w >> 2 : w, total = n_rows * per;    // loads per row, of the warp's rows
-      const uint32_t inv = per > 1 ? 0xFFFFFFFFu / (uint32_t)per + 1u : 0u;
-      auto row_of = [&](int f) { return per > 1 ? (int)__umulhi((uint32_t)f, inv) : f; };
-      auto valid_of = [&](int rr) { return rr_valid_count(row0 + rr, p.n_k, p.causal, p.causal_offset); };
-      if (vec) {
-#pragma unroll 1
-        for (int f0 = lane; f0 < total; f0 += 8 * 32) {
-          int4 q[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u)
-            q[u] = f0 + u * 32 < total ? __ldg(reinterpret_cast<const int4*>(ids) + f0 + u * 32) : make_int4(-1, -1, -1, -1);
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int rr = row_of(f0 + u * 32), vr = valid_of(rr);
-            const uint32_t map = plane + (uint32_t)rr * pitch * 4u;
-            mark(q[u].x, vr, map); mark(q[u].y, vr, map); mark(q[u].z, vr, map); mark(q[u].w, vr, map);
-          }
-        }
-      } else {
-#pragma unroll 1
-        for (int f0 = lane; f0 < total; f0 += 8 * 32) {
-          int q[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) q[u] = f0 + u * 32 < total ? __ldg(ids + f0 + u * 32) : -1;
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int rr = row_of(f0 + u * 32);
-            mark(q[u], valid_of(rr), plane + (uint32_t)rr * pitch * 4u);
-          }
-        }
-      }
-    }
+    const int row0 = tm * BM + quarter * 32, n_rows = max(0, min(32, p.n_q - row0));
+    bool bad = false;
+    int n_cand = rr_mark_rows<1, 4>(p, j == 0 ? p.routes : p.sentinels, j == 0 ? p.k : p.sw, prob, row0, n_rows,
+                                    maps_q + (j == 0 ? 0u : (uint32_t)words * 4u), pitch * 4u, 0, lane, bad);
     if (p.debug && has && j == 0)
       for (int s = 0; s < p.c; ++s) p.cand_scores[g * p.c + s] = __int_as_float(0x7fc00000);
     consumers_sync();                                        // either thread reads both bitmaps

@@ -6,30 +6,26 @@
 // One CTA owns 128 query rows of one problem (consecutive rows at an anchor; a segment of the
 // compacted refresh list at a relay, Section 4.2) and walks the key chunks in tiles of 64,
 // stopping at the last chunk any of its rows may select.
-//   warp 0    : TMA producer (Kc tiles, 128-byte swizzle, one copy per tile, a 32 KB ring)
+//   warp 0    : TMA producer (Kc tiles, 128-byte swizzle, one copy per tile, a ring of 3)
 //   warp 1    : issues tcgen05.mma (M=128, N=64, K=16) into a ring of 3 TMEM
 //               accumulators; the Qc tile is the MMA's A operand in TMEM
 //   warps 2-9 : selection, TWO THREADS PER QUERY ROW: thread j of a row takes the tiles t with
 //               t % 2 == j (two tcgen05.ld 32x32b hand it the tile's 64 scores of its row).
 // What bounds this kernel is the instruction issue of the selection and the latency of its
 // phases, not the GEMM (which is therefore simply issued twice); everything is laid out so that
-// TWO CTAs fit an SM (113 KB of shared memory, 96 registers, 256 TMEM columns each) and one CTA's
-// latency-bound phases hide behind the other's sweeps, as far as a row's column allows it (see the
-// configurations at the end).
-// 256 x 1024 x 1024, keep 48: 276 us, where four threads per row with one CTA per SM and a sentinel
-// kernel behind it (rr_route_sweep.cu, rr_sentinels.cu) took 350 + 60; 64 x 2048 x 2048, keep 96: 413 us,
-// where the streaming kernel took 521.  Issue slots are 47 % busy, the tensor pipe 13 %, DRAM 9 %.
+// TWO CTAs fit an SM (97 KB of shared memory, 96 registers, 256 TMEM columns each) and one CTA's
+// latency-bound phases hide behind the other's sweeps.  It serves keep = k + max(m, 1) <= 28; more kept chunks make its
+// phases so long that four threads per row are better (rr_route_quad.cuh; the figures are there).
 //
 // Sweep 1 (threshold before filtering): scores are cut to bf16 (the upper half of the float, one
-// byte permute per two scores) and each thread keeps packed running maxima of 64 NG groups of
-// columns (64 positions in a tile x NG classes of its tiles): 128 NG groups per row.  The keep-th
+// byte permute per two scores) and each thread keeps packed running maxima of 64 groups of
+// columns (64 positions in a tile): 128 groups per row.  The keep-th
 // largest group maximum, keep = k + max(m, 1), has keep distinct scores of the row at or above it:
-// a valid lower bound tau of the row's keep-th largest score (about 1.25 keep scores pass it).  The
+// a valid lower bound tau of the row's keep-th largest score (about 1.1 keep scores pass it).  The
 // maxima are sorted in registers, two lists at a time (packed compare-exchange); each thread takes
 // its share of keep from the top of its own two lists (binary search), and the shares are shifted
-// twice towards the thread that has more above the lower of the two bounds.  Any shares give a
-// valid bound; these are close to the exact rank (58.9 instead of 58.2 survivors of 1024 random
-// scores at keep = 48; 64.3 with even shares) and follow the data when one thread's tiles hold
+// once towards the thread that has more above the lower of the two bounds.  Any shares give a
+// valid bound; these are close to the exact rank and follow the data when one thread's tiles hold
 // most of the row's best chunks.
 // Sweep 2: each thread appends its scores >= tau as {score, chunk id} to the row's column of CAP
 // entries in shared memory, thread 0 upwards from the bottom, thread 1 downwards from the top.
@@ -46,10 +42,12 @@
 // bounded.
 #include "rr_common.cuh"
 #include "rr_networks.cuh"
+#include "rr_route_select.cuh"
 #include "rr_sm100.cuh"
 #include "rr_warp_topk.cuh"
 
 using namespace sm100;
+using namespace rr_select;
 
 namespace {
 
@@ -58,9 +56,9 @@ constexpr int TPR = 2, SLICE = 32;                 // threads per row, columns p
 constexpr int SEL_WARPS = TPR * (BM / 32);
 constexpr int NT = (2 + SEL_WARPS) * 32;
 constexpr int TMEM_COLS = 256, A_COL = ACC_STAGES * BN;   // Qc tile behind the accumulators
+constexpr int MAX_KEEP = 28;                       // largest k + max(m, 1) that a column of 48 entries serves
 constexpr int MAX_STAGES = ACC_STAGES;             // of the Kc ring: tiles of 16 KB (d = 128) or 8 KB (d = 64)
 constexpr int MAX_HARD = 24;                       // score rows held at once by the slow path
-constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr uint32_t SLOT_PITCH = BM * 8;            // bytes between entries of a row's column
 constexpr uint32_t WORD_PITCH = BM * 4;            // [word][row] areas
 
@@ -81,89 +79,6 @@ __device__ __forceinline__ void quarter_sync(int quarter) {
   asm volatile("bar.sync %0, 64;" ::"r"(quarter + 1) : "memory");
 }
 
-// ---- packed compare-exchanges -----------------------------------------------------------------
-struct DescBF2 {                     // two bf16 lists at a time
-  static __device__ __forceinline__ void ce(uint32_t& a, uint32_t& b) {
-    uint32_t hi, lo;
-    asm("max.bf16x2 %0, %1, %2;" : "=r"(hi) : "r"(a), "r"(b));
-    asm("min.bf16x2 %0, %1, %2;" : "=r"(lo) : "r"(a), "r"(b));
-    a = hi; b = lo;
-  }
-};
-// Non-negative integers below the pattern of +inf, compared as floats: an FMNMX pair per
-// compare-exchange, where unsigned min / max become a compare and two selects.
-struct DescPos {
-  static __device__ __forceinline__ void ce(uint32_t& a, uint32_t& b) {
-    const float hi = fmaxf(__uint_as_float(a), __uint_as_float(b)), lo = fminf(__uint_as_float(a), __uint_as_float(b));
-    a = __float_as_uint(hi); b = __float_as_uint(lo);
-  }
-};
-struct AscPos {
-  static __device__ __forceinline__ void ce(uint32_t& a, uint32_t& b) { DescPos::ce(b, a); }
-};
-struct AscU2 {                       // two lists of 16-bit values at a time
-  static __device__ __forceinline__ void ce(uint32_t& a, uint32_t& b) {
-    const uint32_t hi = __vmaxu2(a, b), lo = __vminu2(a, b);
-    a = lo; b = hi;
-  }
-};
-__host__ __device__ constexpr int pow2_at_least(int n) { int p = 1; while (p < n) p *= 2; return p; }
-
-// ---- rank search over two descending lists ----------------------------------------------------
-// How many entries of the first list belong to the T largest of both (0 <= T <= 2 M): A(i) / B(i)
-// are the lists' values, M entries each.
-template <int M, class FA, class FB>
-__device__ __forceinline__ int rank_split(int T, FA&& A, FB&& B) {
-  int lo = max(0, T - M), hi = min(T, M);
-#pragma unroll 1
-  for (int s = 1; s <= M; s *= 2) {
-    const int mid = (lo + hi) >> 1;
-    const bool more = A(min(mid, M - 1)) > B(min(max(T - mid - 1, 0), M - 1));
-    const bool go = lo < hi;
-    lo = go && more ? mid + 1 : lo;
-    hi = go && !more ? mid : hi;
-  }
-  return lo;
-}
-
-// ---- fixed-point image of a survivor ------------------------------------------------------------
-// Bits of 2^23 + q, q = round(8355000 * sat((s - tau) * scale + 2^-22)): monotone in s, q >= 1 for
-// s >= tau, 0 for an empty slot (-inf); 256 q + slot stays below the pattern of +inf.
-__device__ __forceinline__ uint32_t fixed_bits(float s, float tau, float scale) {
-  float t;
-  asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(t) : "f"(s - tau), "f"(scale), "f"(1.0f / 4194304.0f));
-  return __float_as_uint(fmaf(t, 8355000.0f, 8388608.0f));
-}
-
-__device__ __forceinline__ void tmem_ld_cols(uint32_t a, uint32_t (&r)[32]) { tmem_ld_32x32(a, r); }
-__device__ __forceinline__ void tmem_ld_cols(uint32_t a, uint32_t (&r)[16]) { tmem_ld_32x16(a, r); }
-
-// ---- threshold filter of sweep 2 ------------------------------------------------------------
-// One score: if it passes, {score, chunk id} goes to [w] and w moves on by one entry (a compare,
-// an id add and three predicated instructions; EDGE: ids >= v never pass, one compare more).  Two
-// 4-byte stores: an 8-byte store wants its operands in a register pair, which the scores of a TMEM
-// load are not, and the moves cost more than the second store.
-template <int I, bool EDGE>
-__device__ __forceinline__ void filter_one(uint32_t& w, uint32_t sbits, float tau, uint32_t col0, uint32_t step, int v) {
-  if constexpr (!EDGE) {
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 c;\n\t"
-                 "setp.ge.f32 p, %1, %2;\n\t"
-                 "add.u32 c, %3, %4;\n\t"
-                 "@p st.shared.b32 [%0], %1;\n\t"
-                 "@p st.shared.b32 [%0+4], c;\n\t"
-                 "@p add.u32 %0, %0, %5;\n\t}"
-                 : "+r"(w) : "f"(__uint_as_float(sbits)), "f"(tau), "r"(col0), "n"(I), "r"(step) : "memory");
-  } else {
-    asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b32 c;\n\t"
-                 "add.u32 c, %3, %4;\n\t"
-                 "setp.lt.s32 q, c, %6;\n\t"
-                 "setp.ge.and.f32 p, %1, %2, q;\n\t"
-                 "@p st.shared.b32 [%0], %1;\n\t"
-                 "@p st.shared.b32 [%0+4], c;\n\t"
-                 "@p add.u32 %0, %0, %5;\n\t}"
-                 : "+r"(w) : "f"(__uint_as_float(sbits)), "f"(tau), "r"(col0), "n"(I), "r"(step), "r"(v) : "memory");
-  }
-}
 template <int I, bool EDGE>
 __device__ __forceinline__ void filter_all(uint32_t& w, const uint32_t (&acc)[SLICE], float tau, uint32_t col0,
                                            uint32_t step, int v) {
@@ -228,17 +143,15 @@ __device__ unsigned long long g_rows_phase[32];
 #define PH_LAP(i) do {} while (0)
 #endif
 
-// NG: classes of a thread's tiles (128 NG groups of columns per row); CAP: entries per row.
-template <int D, int NG, int CAP, int CTAS, int STAGES, int ROUNDS>
-__global__ void __launch_bounds__(NT, CTAS)
+constexpr int CAP = 48, STAGES = ACC_STAGES;         // entries of a row's column, tiles of the Kc ring
+template <int D>
+__global__ void __launch_bounds__(NT, 2)
 route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
                   const __grid_constant__ CUtensorMap tmap_k, const int32_t* __restrict__ row_list_arg,
                   uint32_t layer, int hooks, int ring_bytes, int cta_stride) {
   constexpr int KH = D / 64;                               // K-halves of a tile
   constexpr int TILE = BN * D * 2;
-  static_assert(STAGES >= 2 && STAGES <= ACC_STAGES, "see produce()");
   constexpr int M = CAP / 2;                               // entries per half column
-  constexpr int S1 = NG == 2 && CTAS == 2 ? 16 : SLICE;    // columns per load of sweep 1 (64 maxima and 96 registers: no room for 32 scores)
   extern __shared__ __align__(1024) uint8_t smem_raw[];    // (checked below: the swizzle needs it)
   uint8_t* smem = smem_raw;
   uint8_t* sB = smem;                                      // Kc ring; after the sweeps: keys, bitmap
@@ -468,54 +381,38 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
     float tau;
     float scale;
     {
-      uint32_t mx[NG * 32];
+      uint32_t mx[32];
 #pragma unroll
-      for (int i = 0; i < NG * 32; ++i) mx[i] = 0xff80ff80u;
+      for (int i = 0; i < 32; ++i) mx[i] = 0xff80ff80u;
 #pragma unroll 1
-      for (int t0 = j; t0 < n_tiles; t0 += TPR * NG) {
+      for (int t = j; t < n_tiles; t += TPR) {
+        if (!tile_wait(t)) break;
 #pragma unroll
-        for (int c = 0; c < NG; ++c) {
-          const int t = t0 + TPR * c;
-          if (t < n_tiles && tile_wait(t)) {
+        for (int h = 0; h < BN / SLICE; ++h) {
+          const int col0 = t * BN + h * SLICE;
+          uint32_t acc[SLICE];
+          if (col0 < vmaxw) tmem_ld_32x32(acc_addr(t, h), acc);
+          if (h == BN / SLICE - 1) tile_release(t);
+          if (col0 + SLICE <= vminw) {
 #pragma unroll
-            for (int h = 0; h < BN / S1; ++h) {
-              const int col0 = t * BN + h * S1;
-              uint32_t acc[S1];
-              if (col0 < vmaxw) tmem_ld_cols(acc_lane + (uint32_t)((t % ACC_STAGES) * BN + h * S1), acc);
-              if (h == BN / S1 - 1) tile_release(t);
-              if (col0 + S1 <= vminw) {
+            for (int i = 0; i < SLICE / 2; ++i) {
+              const uint32_t pk = __byte_perm(acc[2 * i], acc[2 * i + 1], 0x7632);   // upper halves: bf16, cut
+              asm("max.bf16x2 %0, %0, %1;" : "+r"(mx[h * (SLICE / 2) + i]) : "r"(pk));
+            }
+          } else if (col0 < vmaxw) {                         // some row's last chunk lies inside
+            const int nv = v - col0;
 #pragma unroll
-                for (int i = 0; i < S1 / 2; ++i) {
-                  const uint32_t pk = __byte_perm(acc[2 * i], acc[2 * i + 1], 0x7632);   // upper halves: bf16, cut
-                  asm("max.bf16x2 %0, %0, %1;" : "+r"(mx[c * 32 + h * (S1 / 2) + i]) : "r"(pk));
-                }
-              } else if (col0 < vmaxw) {                     // some row's last chunk lies inside
-                const int nv = v - col0;
-#pragma unroll
-                for (int i = 0; i < S1 / 2; ++i) {
-                  const uint32_t pk = __byte_perm(acc[2 * i], acc[2 * i + 1], 0x7632);
-                  const uint32_t pm = 2 * i + 1 < nv ? pk : (pk & 0xffffu) | 0xff800000u;
-                  asm("max.bf16x2 %0, %0, %1;" : "+r"(mx[c * 32 + h * (S1 / 2) + i]) : "r"(2 * i < nv ? pm : 0xff80ff80u));
-                }
-              }
+            for (int i = 0; i < SLICE / 2; ++i) {
+              const uint32_t pk = __byte_perm(acc[2 * i], acc[2 * i + 1], 0x7632);
+              const uint32_t pm = 2 * i + 1 < nv ? pk : (pk & 0xffffu) | 0xff800000u;
+              asm("max.bf16x2 %0, %0, %1;" : "+r"(mx[h * (SLICE / 2) + i]) : "r"(2 * i < nv ? pm : 0xff80ff80u));
             }
           }
         }
       }
       PH_LAP(0);
-      // two sorted lists of 32 (the halves of mx[0..32)); with two classes the upper half of each
-      // pair of lists is kept: fewer groups than there are, a valid bound all the same
+      // two sorted lists of 32
       OESort<0, 32, DescBF2, 32>::run(mx);
-      if constexpr (NG == 2) {
-        OESort<0, 32, DescBF2, 32>::run(mx + 32);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) asm("max.bf16x2 %0, %0, %1;" : "+r"(mx[i]) : "r"(mx[63 - i]));
-#pragma unroll
-        for (int h = 16; h >= 1; h >>= 1)
-#pragma unroll
-          for (int i = 0; i < 32; ++i)
-            if ((i & h) == 0) DescBF2::ce(mx[i], mx[i + h]);
-      }
       // published in this thread's (still unused) half of the column: list A in the low halves of
       // the words, list B in the high halves, two words to a slot
       const uint32_t pub = col + (uint32_t)(j * M) * SLOT_PITCH;
@@ -530,47 +427,43 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
         const float la = A(max(a - 1, 0)), lb = B(max(b - 1, 0));
         return fminf(a > 0 ? la : pinf, b > 0 ? lb : pinf);
       };
-      // shares in proportion to the threads' non-empty groups (64 NG at most), of which a thread has
-      // kept the g0 / g1 largest maxima
+      // shares in proportion to the threads' non-empty groups (64 at most)
       const int q = v / BN, rem = v % BN;
-      const int c0 = min(64 * NG, ((q + 1) / 2) * BN + ((q & 1) == 0 ? rem : 0)), g0 = min(64, c0);
-      const int c1 = min(64 * NG, (q / 2) * BN + ((q & 1) == 1 ? rem : 0)), g1 = min(64, c1);
-      int share0 = c1 == 0 ? T : c1 == 64 * NG ? (T + 1) / 2 : (int)((float)(T * c0) / (float)(c0 + c1) + 0.5f);
-      share0 = min(g0, max(share0, T - g1));
+      const int c0 = min(64, ((q + 1) / 2) * BN + ((q & 1) == 0 ? rem : 0));
+      const int c1 = min(64, (q / 2) * BN + ((q & 1) == 1 ? rem : 0));
+      int share0 = c1 == 0 ? T : c1 == 64 ? (T + 1) / 2 : (int)((float)(T * c0) / (float)(c0 + c1) + 0.5f);
+      share0 = min(c0, max(share0, T - c1));
       int share = j == 0 ? share0 : T - share0;
       float bound = share_bound(share);
       // messages: word 0 of the other thread's mail slot = this thread's bound, word 1 = the shift
       const uint32_t mail_in = col + (uint32_t)(j * M + MAIL) * SLOT_PITCH, mail_out = col + (uint32_t)((1 - j) * M + MAIL) * SLOT_PITCH;
       float top = fmaxf(A(0), B(0));
       sts32(mail_out, __float_as_uint(bound));
-#pragma unroll 1
-      for (int round = 0; round < ROUNDS; ++round) {
-        quarter_sync(quarter);
-        const float other = ldsf(mail_in);
-        if (round == 0) {                                    // (the other list is still there)
-          const uint32_t w = lds32(col + (uint32_t)((1 - j) * M) * SLOT_PITCH);
-          top = fmaxf(top, fmaxf(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u)));
-        }
-        // the thread with the higher bound counts its maxima at or above the other one's and takes
-        // half of the surplus
-        int ca = 0, cb = 0;
-#pragma unroll
-        for (int s = 16; s >= 1; s >>= 1) {
-          ca += A(ca + s - 1) >= other ? s : 0;
-          cb += B(cb + s - 1) >= other ? s : 0;
-        }
-        ca += A(ca) >= other ? 1 : 0; cb += B(cb) >= other ? 1 : 0;   // ca, cb <= 31 here
-        int shift = max(0, (ca + cb - share) >> 1);
-        if (j == 1) shift = -shift;
-        if (bound > other) sts32(mail_out + 4u, (uint32_t)shift);
-        quarter_sync(quarter);
-        if (bound < other) shift = (int)lds32(mail_in + 4u);
-        if (bound == other) shift = 0;
-        share0 = min(min(g0, T), max(share0 + shift, max(T - g1, 0)));
-        share = j == 0 ? share0 : T - share0;
-        bound = share_bound(share);
-        sts32(mail_out, __float_as_uint(bound));
+      quarter_sync(quarter);
+      const float other = ldsf(mail_in);
+      {                                                      // (the other list is still there)
+        const uint32_t w = lds32(col + (uint32_t)((1 - j) * M) * SLOT_PITCH);
+        top = fmaxf(top, fmaxf(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u)));
       }
+      // the thread with the higher bound counts its maxima at or above the other one's and takes
+      // half of the surplus
+      int ca = 0, cb = 0;
+#pragma unroll
+      for (int s = 16; s >= 1; s >>= 1) {
+        ca += A(ca + s - 1) >= other ? s : 0;
+        cb += B(cb + s - 1) >= other ? s : 0;
+      }
+      ca += A(ca) >= other ? 1 : 0; cb += B(cb) >= other ? 1 : 0;   // ca, cb <= 31 here
+      int shift = max(0, (ca + cb - share) >> 1);
+      if (j == 1) shift = -shift;
+      if (bound > other) sts32(mail_out + 4u, (uint32_t)shift);
+      quarter_sync(quarter);
+      if (bound < other) shift = (int)lds32(mail_in + 4u);
+      if (bound == other) shift = 0;
+      share0 = min(min(c0, T), max(share0 + shift, max(T - c1, 0)));
+      share = j == 0 ? share0 : T - share0;
+      bound = share_bound(share);
+      sts32(mail_out, __float_as_uint(bound));
       // the lists are done with: the half column is cleared (empty slots read as -inf in the sort), the
       // mail slot once its last message has been read
 #pragma unroll
@@ -737,69 +630,14 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
       const int m0 = go ? n0 : 0, m1 = go ? n1 : 0;
       if (width > 0) {
         if (width <= 16) gather_ids<16>(col, e0, m0, e1, m1, bits, sampling, dst, width, vec, go);
-        else if (width <= 32) gather_ids<32>(col, e0, m0, e1, m1, bits, sampling, dst, width, vec, go);
-        else if (NG == 1 || CTAS == 2 || width <= 64) gather_ids<64>(col, e0, m0, e1, m1, bits, sampling, dst, width, vec, go);
-        else if constexpr (NG > 1 && CTAS == 1) gather_ids<128>(col, e0, m0, e1, m1, bits, sampling, dst, width, vec, go);
+        else gather_ids<32>(col, e0, m0, e1, m1, bits, sampling, dst, width, vec, go);
       }
     }
     PH_LAP(6);
     if (sampling) quarter_sync(quarter);                     // the bitmap is complete
     // ===== sentinels (Section 3.1 items 2, 3): the row's second thread ===================================
-    // pool <= r: the whole pool in ascending order; else for t = 0, 1, ...: j = floor(u_t v / 2^32),
-    // accept iff j is not excluded and not drawn yet; after 64 r draws the smallest free chunks.
-    // The ids are collected in the score words of the row's column (done with) and go out with
-    // 16-byte stores.
-    if (j == 1 && sampling && go) {
-      int pool = v - n_excl;
-      auto word = [&](int id) -> uint32_t { return bits + (uint32_t)(id >> 5) * WORD_PITCH; };
-      if (p.n_global) {           // mandatory global sentinels: a slot each after the random ones
-        int32_t* glob = sent + p.m + p.r;
-        int gi = 0;
-        for (int b = 0; b < 2; ++b) {
-          if (!((p.global_mask >> b) & 1)) continue;
-          const int id = b == 0 ? 0 : v - 1;
-          const uint32_t w = lds32(word(id)), bit = 1u << (id & 31);
-          const bool free_ = !(w & bit);
-          if (free_) { sts32(word(id), w | bit); --pool; }
-          glob[gi++] = free_ ? id : -1;
-        }
-      }
-      int32_t* rnd = sent + p.m;
-      const bool staged = p.r <= CAP && ((p.m | p.r | p.sw) & 3) == 0;
-      const uint32_t stage = col;
-      auto put = [&](int slot, int id) { if (staged) sts32(stage + (uint32_t)slot * SLOT_PITCH, (uint32_t)id); else rnd[slot] = id; };
-      int taken = 0;
-      if (p.r > 0 && pool > 0) {
-        if (pool > p.r) {
-          const unsigned long long rk = rr_row_key(p.seed, (uint32_t)g);
-          const int limit = 64 * p.r;
-          // four draws are generated at a time (independent 64-bit mixes overlap); they are still
-          // accepted strictly in draw order
-#pragma unroll 1
-          for (int t0 = 0; t0 < limit && taken < p.r; t0 += 4) {
-            int j4[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-              j4[i] = (int)__umulhi(rr_draw_u32(rk, layer, (uint32_t)(t0 + i)), (uint32_t)v);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const bool live = (t0 + i < limit) & (taken < p.r);
-              const uint32_t w = lds32(word(j4[i])), bit = 1u << (j4[i] & 31);
-              if (live && !(w & bit)) { sts32(word(j4[i]), w | bit); put(taken++, j4[i]); }
-            }
-          }
-        }
-        // whole pool (pool <= r) or the bounded-work fill: smallest free chunks first
-        for (int id = 0; id < v && taken < p.r; ++id)
-          if (!((lds32(word(id)) >> (id & 31)) & 1u)) put(taken++, id);
-      }
-      for (int e = taken; e < p.r; ++e) put(e, -1);
-      if (staged)
-        for (int e = 0; e < p.r; e += 4)
-          *reinterpret_cast<int4*>(rnd + e) =
-              make_int4((int)lds32(stage + (uint32_t)e * SLOT_PITCH), (int)lds32(stage + (uint32_t)(e + 1) * SLOT_PITCH),
-                        (int)lds32(stage + (uint32_t)(e + 2) * SLOT_PITCH), (int)lds32(stage + (uint32_t)(e + 3) * SLOT_PITCH));
-    }
+    if (j == 1 && sampling)
+      draw_sentinels<WORD_PITCH, SLOT_PITCH, CAP>(p, bits, col, g, v, n_excl, layer, lane, go);
     PH_LAP(7);
   }
 
@@ -879,73 +717,24 @@ route_rows_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   if (!row_list_arg) rr_pdl_wait();                        // complete only after the predecessor is
 }
 
-// ---- configurations ------------------------------------------------------------------------------
-// keep = k + max(m, 1) and the number of key chunks decide how many entries a row's column needs: with
-// 64 groups to a thread and class the bound lets 1.05-1.25 keep scores pass (few where a group holds
-// one chunk or two).  A row that needs more takes the slow path, and the CTA that meets one runs 12 us
-// longer (a column of 76 entries at keep 48 let 7 in 10^5 rows of 1024 chunks through: 289 instead of
-// 265 us on 2048 CTAs); a longer column than needed lengthens the sorts (keep 32, 256 x 1024 x 1024:
-// 64 entries 247 us, 80 entries 271 us; keep 80, 64 x 2048 x 2048: 128 entries 384, 152 entries 406).
-// What counts most is whether two CTAs fit an SM: 80 entries are the longest column that lets them
-// (88 at d = 64).
-//   keep <= 48: 128 groups (mean / largest of 10^5 random rows of 1024 chunks: keep 24 27 / 40, keep 36
-//               41 / 55, keep 48 59 / 80);
-//   beyond:     256 groups, whose maxima alone are 64 registers of a thread: sweep 1 then takes 16 scores
-//               at a time where two CTAs leave it 96 registers.
-// MOST: most kept chunks for a column of 80, 88 (d = 64), 104 or 128 entries, by the number of key chunks.  The
-// lines lie where fewer than 1 row in 10^4 needs more, over random and clustered rows of every length up
-// to n_k (largest of 99.98 % of them: keep 70 of 256 chunks 77, keep 62 of 512 77, keep 58 of 1024 76,
-// keep 56 of 2048 75); rows of 161 to 200 chunks (three and a bit tiles) are the worst of their length.
-// 9 layers at rho = 0.2, two CTAs of 80 or 88 entries against one of 104 or 128 entries:
-//   256 x 256 x 256, keep 65: 1189 and 1874 us; 200 x 140 x 1024, keep 58: 959 and 1059; 64 x 2048 x 2048,
-//   keep 56: 2495 and 3171; 128 x 512 x 512 (d 64), keep 68: 1140 and 1679.
-// Past a line the slow path costs more than the second CTA gives: 40 x 500 x 450, keep 66 at rho = 0.004 514
-// us with one CTA, 636 with two; 100 x 300 x 2048 (d 64), keep 60: 887 and 1380.  Shorter columns where one
-// CTA runs: 256 x 256 x 256, keep 80 of 104 entries instead of 128 1793 and 1889 us, keep 88 of 128 instead of
-// 144 1950 and 2043; 200 x 140 x 1024, keep 88 of 128 instead of 144 entries, past the line of 84: 1829 and 1633.
-struct Plan { int variant, ctas, ring_bytes; size_t smem; };   // ctas: per SM
-constexpr int VARIANTS = 8, CAPS[VARIANTS] = {48, 64, 80, 80, 88, 104, 128, 144};
-constexpr struct { int n_k, cap80, cap88, cap104, cap128; } MOST[] = {
-    {256, 70, 76, 80, 92}, {320, 66, 72, 80, 84}, {512, 62, 68, 76, 84}, {1024, 58, 64, 70, 84},
-    {1536, 56, 62, 64, 80}, {2048, 56, 0, 64, 80}, {RR_MAX_NK, 0, 0, 64, 80}};   // (0: the bitmaps leave no room for two)
-
+// ---- configuration -------------------------------------------------------------------------------
+// 48 entries hold what passes the bound (keep 24: mean / largest of 10^5 random rows of 1024 chunks 27 / 40); a row that
+// needs more takes the slow path, and the CTA that meets one runs 12 us longer.
+struct Plan { int ctas, ring_bytes; size_t smem; };   // ctas: per SM
 bool plan(const RRParams& p, Plan& out) {
   const int keep = p.k + (p.m > 0 ? p.m : 1);
-  if (p.dtype != RR_BF16 || (p.d != 64 && p.d != 128) || p.n_k > RR_MAX_NK || keep > 96) return false;
-  if (keep <= 48) {
-    out.variant = keep <= 28 ? 0 : keep <= 36 ? 1 : 2;
-  } else {
-    int i = 0;
-    while (p.n_k > MOST[i].n_k) ++i;
-    const auto& most = MOST[i];
-    const bool narrow = p.k <= 64 && p.m <= 64;      // (with 96 registers a thread orders 64 ids at most)
-    // 88 entries fit twice at d = 64 only, where the Kc tiles are smaller; they spill a few registers and
-    // gain nothing where every CTA has an SM to itself (3 x 489 x 489, keep 53: 88 entries 531 us, 104
-    // entries with one CTA per SM 525, 80 entries 518)
-    out.variant = narrow && keep <= most.cap80 ? 3 : narrow && p.d == 64 && keep <= most.cap88 && p.n_tiles > rr_sm_count() ? 4
-                  : keep <= most.cap104 ? 5 : keep <= most.cap128 ? 6 : 7;
-  }
+  if (p.dtype != RR_BF16 || (p.d != 64 && p.d != 128) || p.n_k > RR_MAX_NK || keep > MAX_KEEP) return false;
   const int words = (p.n_k + 31) / 32;
-  const int stages = p.d == 64 || (out.variant != 2 && out.variant != 3) ? 3 : 2;
-  int ring = stages * BN * p.d * 2;
+  int ring = STAGES * BN * p.d * 2;
   if (ring < words * (int)WORD_PITCH) ring = words * (int)WORD_PITCH;
   out.ring_bytes = (ring + 1023) / 1024 * 1024;
-  out.smem = (size_t)out.ring_bytes + CTL_BYTES + (size_t)CAPS[out.variant] * SLOT_PITCH;
-  out.ctas = out.variant <= 4 && 2 * (out.smem + 1024) <= 228 * 1024 ? 2 : 1;
+  out.smem = (size_t)out.ring_bytes + CTL_BYTES + (size_t)CAP * SLOT_PITCH;
+  out.ctas = 2 * (out.smem + 1024) <= 228 * 1024 ? 2 : 1;
   return out.smem <= 227 * 1024;
 }
 
 typedef void (*Kernel)(RRParams, const __nv_bfloat16*, const CUtensorMap, const int32_t*, uint32_t, int, int, int);
-Kernel kernel_of(int d, int variant) {
-  static const Kernel table[2][VARIANTS] = {
-      {route_rows_kernel<64, 1, 48, 2, 3, 1>, route_rows_kernel<64, 1, 64, 2, 3, 2>, route_rows_kernel<64, 1, 80, 2, 3, 2>,
-       route_rows_kernel<64, 2, 80, 2, 3, 2>, route_rows_kernel<64, 2, 88, 2, 3, 2>, route_rows_kernel<64, 2, 104, 1, 3, 1>,
-       route_rows_kernel<64, 2, 128, 1, 3, 1>, route_rows_kernel<64, 2, 144, 1, 3, 1>},
-      {route_rows_kernel<128, 1, 48, 2, 3, 1>, route_rows_kernel<128, 1, 64, 2, 3, 2>, route_rows_kernel<128, 1, 80, 2, 2, 2>,
-       route_rows_kernel<128, 2, 80, 2, 2, 2>, nullptr, route_rows_kernel<128, 2, 104, 1, 3, 1>,
-       route_rows_kernel<128, 2, 128, 1, 3, 1>, route_rows_kernel<128, 2, 144, 1, 3, 1>}};
-  return table[d == 128 ? 1 : 0][variant];
-}
+Kernel kernel_of(int d) { return d == 128 ? route_rows_kernel<128> : route_rows_kernel<64>; }
 
 }  // namespace
 
@@ -972,18 +761,15 @@ cudaError_t rr_launch_route_rows(const RRParams& p, const void* qc, const void* 
   if (e != cudaSuccess) return e;
   static unsigned long long attr_done = 0;      // devices on which the attributes are set
   e = rr_once_per_device(attr_done, [] {
-    for (int d = 64; d <= 128; d += 64)
-      for (int v = 0; v < VARIANTS; ++v) {
-        if (!kernel_of(d, v)) continue;
-        const cudaError_t a = cudaFuncSetAttribute((const void*)kernel_of(d, v),
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-        if (a != cudaSuccess) return a;
-        cudaFuncSetAttribute((const void*)kernel_of(d, v), cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-      }
+    for (int d = 64; d <= 128; d += 64) {
+      const cudaError_t a = cudaFuncSetAttribute((const void*)kernel_of(d), cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+      if (a != cudaSuccess) return a;
+      cudaFuncSetAttribute((const void*)kernel_of(d), cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    }
     return cudaSuccess;
   });
   if (e != cudaSuccess) return e;
-  e = rr_launch_pdl(kernel_of(p.d, pl.variant), p.n_tiles, NT, pl.smem, st, p, (const __nv_bfloat16*)qc, tmap, row_list,
+  e = rr_launch_pdl(kernel_of(p.d), p.n_tiles, NT, pl.smem, st, p, (const __nv_bfloat16*)qc, tmap, row_list,
                     (uint32_t)layer, hooks, pl.ring_bytes, pl.ctas * rr_sm_count());
   rr_count_launch();
   return e;
