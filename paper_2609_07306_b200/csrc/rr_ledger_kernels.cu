@@ -18,8 +18,7 @@ constexpr unsigned FULL = 0xFFFFFFFFu;
 // per-layer counters: nothing later in the layer reads either.
 __global__ void __launch_bounds__(RR_ROW_TILE)
 compact_kernel(RRParams p, unsigned long long dense_pairs) {
-  __shared__ int s_part[RR_ROW_TILE / 32];
-  __shared__ int s_base;
+  __shared__ int s_part[RR_ROW_TILE / 32], s_cnt[RR_ROW_TILE / 32];   // earlier tiles' counts, by warp; this tile's
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tile_id = blockIdx.x;
   const int prob = tile_id / p.tiles_per_problem, tile = tile_id % p.tiles_per_problem;
@@ -56,31 +55,28 @@ compact_kernel(RRParams p, unsigned long long dense_pairs) {
     return;
   }
 
-  int part = 0;
-  for (int t = tid; t < tile_id; t += RR_ROW_TILE) part += p.tile_counts[t];
-#pragma unroll
-  for (int off = 16; off; off >>= 1) part += __shfl_xor_sync(FULL, part, off);
-  if (lane == 0) s_part[warp] = part;
-  __syncthreads();
-  if (tid == 0) {
-    int b = 0;
-    for (int w = 0; w < RR_ROW_TILE / 32; ++w) b += s_part[w];
-    s_base = b;
-  }
-  __syncthreads();
-  const int base = s_base;
-  __syncthreads();
-
+  // The row's flag and age are asked for together with the counts (one round trip to L2), and one barrier
+  // serves the base and the places inside the tile: 256 x 256 rows, 24 layers 938 -> 925 us.
   const int i = tile * RR_ROW_TILE + tid;
   const int g = prob * p.n_q + i;
-  const bool f = (i < p.n_q) && p.flags[g] != 0;
+  const bool in = i < p.n_q;
+  const bool f = in && p.flags[g] != 0;
+  const int age = in ? p.ages[g] : 0;
+  int part = 0;
+  for (int t = tid; t < tile_id; t += RR_ROW_TILE) part += p.tile_counts[t];
+  part = __reduce_add_sync(FULL, part);
   const unsigned bal = __ballot_sync(FULL, f);
-  if (lane == 0) s_part[warp] = __popc(bal);
+  if (lane == 0) { s_part[warp] = part; s_cnt[warp] = __popc(bal); }
   __syncthreads();
-  int before = 0;
-  for (int w = 0; w < warp; ++w) before += s_part[w];
+  int base = 0, before = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < RR_ROW_TILE / 32; ++w) {
+    base += s_part[w];
+    if (w < warp) before += s_cnt[w];
+    total += s_cnt[w];
+  }
   if (f) p.refresh_rows[base + before + __popc(bal & ((1u << lane) - 1u))] = g;
-  if (i < p.n_q) p.ages[g] = f ? 0 : p.ages[g] + 1;
+  if (in) p.ages[g] = f ? 0 : age + 1;
   if (tid == 0) {
     if (tile_id == 0) {
       p.counters[RR_CNT_LAYER_CALLS] += 1;
@@ -89,8 +85,7 @@ compact_kernel(RRParams p, unsigned long long dense_pairs) {
     }
     if (tile == 0) p.problem_offsets[prob] = base;
     if (tile_id == p.n_tiles - 1) {
-      int total = base;
-      for (int w = 0; w < RR_ROW_TILE / 32; ++w) total += s_part[w];
+      total += base;
       p.problem_offsets[p.P] = total;
       *p.refresh_count = total;
       if (p.force_threshold > 0) {    // this call was tested: decide about the next ones
