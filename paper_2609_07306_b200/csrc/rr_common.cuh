@@ -69,9 +69,9 @@ struct rr_ledger {
 
 // ---- device helpers -------------------------------------------------------------------
 __host__ __device__ __forceinline__ int rr_valid_count(int i, int n_k, int causal, int off) {
-  if (!causal) return n_k;
-  long long v = (long long)i + 1 + off;
-  return v > n_k ? n_k : (v < 0 ? 0 : (int)v);
+  // (an offset beyond n_k gives every row all chunks; 32 bits are enough then)
+  const int o = off < n_k ? off : n_k, v = i + 1 + o;
+  return !causal || v > n_k ? n_k : v;
 }
 
 // Monotone map float -> uint32 (larger float <=> larger key); -0.0 is folded onto +0.0.

@@ -230,7 +230,7 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   constexpr int TMEM_COLS = CTAS == 2 ? 256 : 512;
   constexpr int XCH = CTAS == 2 ? 96 : 256;                // second set of columns for the exchanges (first: 0, over the accumulators)
   static_assert(CAP % (2 * TPR) == 0 && TPR * M <= (CTAS == 2 ? 96 : 192), "exchange columns");
-  constexpr int S1 = NG == 2 && CTAS == 2 ? 8 : 16;        // columns per load of sweep 1
+  constexpr int S1 = 16;                                   // columns per load of sweep 1
   extern __shared__ __align__(1024) uint8_t smem_raw[];    // (checked below: the swizzle needs it)
   uint8_t* smem = smem_raw;
   uint8_t* sB = smem;                                      // Kc ring; after the sweeps: keys, bitmap
@@ -264,6 +264,11 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   // book-keeping that is not read here, and has triggered after its own wait: the inputs are complete.
   // The wait for it is then at the end of every path (see rr_pdl_wait).
   if (TEST || row_list_arg) rr_pdl_wait();
+  // The list's length and this problem's part of it are asked for together: the rows hang on them, and the Qc rows
+  // on those.
+  const int prob = blockIdx.x % p.P;
+  int list_n = 0, list_lo = 0, list_hi = 0;
+  if (row_list_arg) { list_n = *p.refresh_count; list_lo = p.problem_offsets[prob]; list_hi = p.problem_offsets[prob + 1]; }
   // a relay call that the forced-anchor policy turned into full routing has the identity list:
   // take the anchor's path (consecutive rows, no gathers through the list)
   const bool forced_call = row_list_arg && p.force_threshold > 0 && p.force_in[0] > 0;
@@ -271,16 +276,14 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   // rows that are not on it masked out: gathering 7/8 of the rows through the list costs more
   // than sweeping the missing eighth for nothing (results per row are the same either way).
   const bool dense_refresh = row_list_arg && !forced_call &&
-                             (long long)(*p.refresh_count) * 8 >= (long long)p.rows * 7;
+                             (long long)list_n * 8 >= (long long)p.rows * 7;
   const int32_t* __restrict__ row_list = (forced_call || dense_refresh) ? nullptr : row_list_arg;
   const bool force_hard = hooks & 1, force_timeout = hooks & 2;      // test hooks
   // Row tiles are handed out heaviest first (under the causal mask the last tile of a problem
   // walks the most key chunks), so the tail of the grid is made of the short ones and, where a refresh
   // list is short, of the CTAs that find no tile: in front they kept the SMs from the
   // others (17 % of 256 x 1024 rows on the list: 130 -> 120 us).
-  const int prob = blockIdx.x % p.P;
-  int seg_lo = 0, seg_hi = p.n_q;
-  if (row_list) { seg_lo = p.problem_offsets[prob]; seg_hi = p.problem_offsets[prob + 1]; }
+  const int seg_lo = row_list ? list_lo : 0, seg_hi = row_list ? list_hi : p.n_q;
   const int tm = (seg_hi - seg_lo + BM - 1) / BM - 1 - (int)(blockIdx.x / p.P);
   if (tm < 0) { if (!TEST && !row_list_arg) rr_pdl_wait(); return; }  // nothing to do (uniform per CTA)
   const bool tested = TEST && !(p.force_threshold > 0 && p.force_in[0] > 0);   // (a forced anchor routes every row)
