@@ -54,7 +54,7 @@
 using namespace sm100;
 using namespace rr_select;
 
-typedef void (*rr_quad_kernel)(RRParams, const __nv_bfloat16*, const CUtensorMap, const int32_t*, uint32_t, int, int, int);
+typedef void (*rr_quad_kernel)(RRParams, const __nv_bfloat16*, const CUtensorMap, const int32_t*, uint32_t, int, int, int, int);
 rr_quad_kernel rr_quad_kernel_d64(int variant, bool test);     // (the kernels of the two head widths are compiled apart)
 rr_quad_kernel rr_quad_kernel_d128(int variant, bool test);
 
@@ -221,7 +221,7 @@ template <int D, int NG, int CAP, int CTAS, bool TEST>
 __global__ void __launch_bounds__(NT, CTAS)
 route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
                   const __grid_constant__ CUtensorMap tmap_k, const int32_t* __restrict__ row_list_arg,
-                  uint32_t layer, int hooks, int ring_bytes, int cta_stride) {
+                  uint32_t layer, int hooks, int ring_bytes, int cta_stride, int rows_per_cta) {
   constexpr int KH = D / 64;                               // K-halves of a tile
   constexpr int TILE = BN * D * 2;
   constexpr int STAGES = stages_of(D, CTAS);
@@ -284,14 +284,16 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   // list is short, of the CTAs that find no tile: in front they kept the SMs from the
   // others (17 % of 256 x 1024 rows on the list: 130 -> 120 us).
   const int seg_lo = row_list ? list_lo : 0, seg_hi = row_list ? list_hi : p.n_q;
-  const int tm = (seg_hi - seg_lo + BM - 1) / BM - 1 - (int)(blockIdx.x / p.P);
+  const int own = TEST ? rows_per_cta : BM;                // rows of a CTA (fewer than the MMA's: the others are empty)
+  const int tm = (seg_hi - seg_lo + own - 1) / own - 1 - (int)(blockIdx.x / p.P);
   if (tm < 0) { if (!TEST && !row_list_arg) rr_pdl_wait(); return; }  // nothing to do (uniform per CTA)
   const bool tested = TEST && !(p.force_threshold > 0 && p.force_in[0] > 0);   // (a forced anchor routes every row)
 
   // row of the CTA's tile -> query row of the problem and global row id; -1 = no row
   auto locate = [&](int rr, int& row_out, int& g_out) {
-    const int local = tm * BM + rr;
+    const int local = tm * own + rr;
     row_out = -1; g_out = 0;
+    if (TEST && rr >= own) return;
     if (row_list) {
       if (seg_lo + local < seg_hi) { g_out = row_list[seg_lo + local]; row_out = g_out - prob * p.n_q; }
     } else if (local < p.n_q) {
@@ -334,7 +336,7 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   // The Kc loads depend on nothing but the number of key tiles (from the tile's last row: rows
   // ascend inside a tile), and the ring's stages are all free: the producer fills the ring before
   // the CTA's first barrier, while the Qc rows are on their way.
-  const int last_local = min(seg_hi - seg_lo, (tm + 1) * BM) - 1;
+  const int last_local = min(seg_hi - seg_lo, (tm + 1) * own) - 1;
   const int last_row = row_list ? row_list[seg_lo + last_local] - prob * p.n_q : last_local;
   const int n_tiles = (rr_valid_count(last_row, p.n_k, p.causal, p.causal_offset) + BN - 1) / BN;
   const uint32_t ring = smem_u32(sB);
@@ -437,9 +439,9 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
       const int nprob = nb % p.P;
       int nlo = 0, nhi = p.n_q;
       if (row_list) { nlo = p.problem_offsets[nprob]; nhi = p.problem_offsets[nprob + 1]; }
-      const int ntm = (nhi - nlo + BM - 1) / BM - 1 - nb / p.P;
-      for (int i = lane; i < BM && ntm >= 0; i += 32) {
-        const int local = ntm * BM + i;
+      const int ntm = (nhi - nlo + own - 1) / own - 1 - nb / p.P;
+      for (int i = lane; i < own && ntm >= 0; i += 32) {
+        const int local = ntm * own + i;
         if (local >= nhi - nlo) break;
         const size_t grow = row_list ? (size_t)row_list[nlo + local] : (size_t)nprob * p.n_q + local;
         const char* src = reinterpret_cast<const char*>(qc + grow * D);
@@ -471,7 +473,7 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
     if (tested) {
       // ---- the ledger rows of the quarter's 32 query rows, read as one array, into the bitmaps -------------
       // (two warps the routes, two the sentinels)
-      const int row0 = tm * BM + quarter * 32, n_rows = max(0, min(32, p.n_q - row0));
+      const int row0 = tm * own + quarter * 32, n_rows = max(0, min(32, p.n_q - row0));
       bool bad = false;
       int n_cand = rr_mark_rows<2, SLOT_PITCH>(p, pair == 0 ? p.routes : p.sentinels, pair == 0 ? p.k : p.sw, prob, row0, n_rows,
                                                smem_u32(s_col) + (uint32_t)quarter * 256u + 4u * (uint32_t)pair, 8u, side, lane, bad);
@@ -622,11 +624,11 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
     // A pair's two threads fill its part from both ends.  Running over into the other pair's part only spoils
     // a row that has overflowed; the two in the middle stop where they would leave the column.
     const uint32_t step = side == 0 ? SLOT_PITCH : 0u - SLOT_PITCH;
-    const uint32_t own = slot(j == 0 ? 0 : j == 1 ? split - 1 : j == 2 ? split : CAP - 1);   // this thread's entry 0
+    const uint32_t first = slot(j == 0 ? 0 : j == 1 ? split - 1 : j == 2 ? split : CAP - 1);   // this thread's entry 0
     const int room = j == 1 ? split : j == 2 ? CAP - split : CAP;
-    uint32_t waddr = own;
+    uint32_t waddr = first;
     bool over = false;                                       // the room did not suffice
-    auto filled = [&]() -> int { return (int)(side == 0 ? waddr - own : own - waddr); };     // bytes
+    auto filled = [&]() -> int { return (int)(side == 0 ? waddr - first : first - waddr); };     // bytes
 #pragma unroll 1
     for (int t = pair; t < n_tiles; t += 2) {
       const int gt = n_tiles + t, col0 = t * BN + side * SLICE;
@@ -651,7 +653,7 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
                 ++n;
               }
             }
-            if (n > room) waddr = own + step * (uint32_t)room, over = true;
+            if (n > room) waddr = first + step * (uint32_t)room, over = true;
           }
         }
       }
@@ -842,7 +844,7 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
       uint32_t* scratch = (uint32_t*)s_col + (size_t)hard_slots * nk_words * 32 + sw * (256 + nk_words);
       for (int hs = sw; hs < hard_slots && done + hs < n_hard; hs += SEL_WARPS) {
         const int rr = ctl->hard_rows[done + hs];
-        const int hg = row_list ? row_list[seg_lo + tm * BM + rr] : prob * p.n_q + tm * BM + rr;
+        const int hg = row_list ? row_list[seg_lo + tm * own + rr] : prob * p.n_q + tm * own + rr;
         const int hv = rr_valid_count(hg - prob * p.n_q, p.n_k, p.causal, p.causal_offset);
         const uint32_t* keys = (const uint32_t*)s_col + (size_t)hs * nk_words * 32;
         warptopk::route_row(p, keys, scratch, scratch + 256, hg, hv, layer, lane);
@@ -869,7 +871,8 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   }
   if (tid == 0 && ctl->abort_flag) atomicOr(p.status, RR_STATUS_TIMEOUT);
   if (tested && tid == 0) {
-    p.tile_counts[prob * p.tiles_per_problem + tm] = (int)ctl->flagged;
+    // (several CTAs may share a tile of the list; the previous call's list kernel left the counts at zero)
+    atomicAdd(&p.tile_counts[prob * p.tiles_per_problem + tm * own / RR_ROW_TILE], (int)ctl->flagged);
     atomicAdd(&p.counters[RR_CNT_FLAGGED_ROWS], (unsigned long long)ctl->flagged);
     atomicAdd(&p.counters[RR_CNT_CAND_PAIRS], (unsigned long long)ctl->cand);
     atomicAdd(&p.counters[RR_CNT_FULL_PAIRS], ctl->full_pairs);
