@@ -92,7 +92,10 @@ typedef struct rr_config {
                               bits 6, 7 (tests): the first wait of the first CTA of the first
                               routing launch (bit 6) / strip rescoring launch (bit 7) of this
                               ledger counts as expired, once: that CTA gives up as after a real
-                              time-out and the status word gets RR_STATUS_TIMEOUT          */
+                              time-out and the status word gets RR_STATUS_TIMEOUT;
+                              bit 9 (tests): the same for a wait that expires while the first
+                              relay whose test runs inside the routing kernel decides about its
+                              rows                                                          */
   /* Optional policies either side of the trigger; all zero = the plain method.             */
   int32_t global_sentinels;/* mandatory global candidates (Section 3.1, item 3): bit 0 = the
                               sink chunk 0, bit 1 = the most recent chunk the row may select.

@@ -212,6 +212,7 @@ int route_layer(rr_ledger* L, const void* qc, const void* kc, int layer, bool an
       // The routing kernel tests every row on the scores of its first sweep; the list is built afterwards.
       int hooks = sweep_hooks(L);
       if (L->timeout_shots & 2) { hooks |= 2; L->timeout_shots &= ~2; }
+      if (L->timeout_shots & 4) { hooks |= 4; L->timeout_shots &= ~4; }
       LAUNCH(RR_KIND_ROUTE_FUSED, rr_launch_route_quad(p, qc, kc, nullptr, true, layer, hooks, st));
       LAUNCH(RR_KIND_COMPACT, rr_launch_compact(p, L->dense_pairs_per_layer, st));
       if (p.chunk_tokens > 0) LAUNCH(RR_KIND_EXPAND, rr_launch_expand(p, 0, st));
@@ -299,7 +300,7 @@ int rr_ledger_init(const rr_config* cfg, void* dev_ledger, size_t ledger_bytes,
   L->dev_scratch = dev_scratch; L->scratch_bytes = scratch_bytes;
   L->export_bytes = lay.export_total;
   L->anchored = 0;
-  L->timeout_shots = (cfg->debug_outputs >> 6) & 3;
+  L->timeout_shots = ((cfg->debug_outputs >> 6) & 3) | ((cfg->debug_outputs >> 7) & 4);
   L->device = -1;
   cudaGetDevice(&L->device);           // informational; failure (no GPU) leaves -1
   cudaGetLastError();

@@ -81,7 +81,8 @@ struct Ctl {
   uint8_t cnt[TPR][BM];                 // survivors per thread; after the cuts [0], [1]: cut k / k + m undecided
   uint8_t hard_rows[BM];                // rows handed to the slow path, in registration order
   int8_t hard_slot[BM];                 // position of a row in hard_rows, -1 = none
-  uint32_t flagged, cand;               // of the test: rows that failed, candidates looked at,
+  uint8_t gave_up[BM / 32];             // of the test: a warp of the quarter has met a wait that gave up,
+  uint32_t flagged, cand;               // rows that failed, candidates looked at,
   unsigned long long full_pairs;        // valid chunks of the rows that failed
 };
 constexpr int CTL_BYTES = 1024;
@@ -253,6 +254,7 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
     ctl->abort_flag = 0;
     ctl->hard_n = 0;
     ctl->flagged = 0; ctl->cand = 0; ctl->full_pairs = 0ull;
+    for (int q = 0; q < BM / 32; ++q) ctl->gave_up[q] = 0;
     mbar_fence_init();
   }
   if ((smem_u32(smem) & 1023u) != 0u) {                    // reported like a wait that gave up
@@ -278,7 +280,7 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   const bool dense_refresh = row_list_arg && !forced_call &&
                              (long long)list_n * 8 >= (long long)p.rows * 7;
   const int32_t* __restrict__ row_list = (forced_call || dense_refresh) ? nullptr : row_list_arg;
-  const bool force_hard = hooks & 1, force_timeout = hooks & 2;      // test hooks
+  const bool force_hard = hooks & 1, force_timeout = hooks & 2, force_late = hooks & 4;      // test hooks
   // Row tiles are handed out heaviest first (under the causal mask the last tile of a problem
   // walks the most key chunks), so the tail of the grid is made of the short ones and, where a refresh
   // list is short, of the CTAs that find no tile: in front they kept the SMs from the
@@ -561,16 +563,23 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
 #pragma unroll
       for (int i = 0; i < LIST; ++i) sts32(slot(TPR * i + j), mx[i]);
       if (tested) { sts32(slot(j) + 4u, __float_as_uint(amin)); sts32(slot(TPR + j) + 4u, __float_as_uint(bmax)); }
+      // Whether the test stands is one decision of the quarter, taken at the barrier: the abort flag may rise at any
+      // time, and warps that read it for themselves could part here, some of them at barriers that the others never
+      // reach.  (A wait that gave up before: the rows stay as they are.  One that gives up later: see tile_wait.)
+      if (tested && lane == 0 && (!alive || *abort_flag != 0u)) ctl->gave_up[quarter] = 1;
       quarter_sync(quarter);
       if (tested) {
+        const bool stands = ctl->gave_up[quarter] == 0;
+        // test hook: a wait expires between the decision and what hangs on it, seen by one warp of the four at first
+        if (force_late && blockIdx.x == 0 && j == TPR - 1) *abort_flag = 1u;
 #pragma unroll
         for (int t = 0; t < TPR; ++t) {
           amin = fminf(amin, ldsf(slot(t) + 4u));
           bmax = fmaxf(bmax, ldsf(slot(TPR + t) + 4u));
         }
-        routed = row >= 0 && *abort_flag == 0u && rr_challenge(p, g, amin, bmax);   // (a wait that gave up: the rows stay)
+        routed = row >= 0 && stands && rr_challenge(p, g, amin, bmax);
         if (j == 0) {
-          if (row >= 0 && *abort_flag == 0u) { p.flags[g] = routed ? 1 : 0; p.alpha[g] = amin; p.beta[g] = bmax; }
+          if (row >= 0 && stands) { p.flags[g] = routed ? 1 : 0; p.alpha[g] = amin; p.beta[g] = bmax; }
           const int n_flag = __popc(__ballot_sync(FULL, routed)), v_sum = __reduce_add_sync(FULL, routed ? v : 0);
           if (lane == 0) { atomicAdd(&ctl->flagged, (uint32_t)n_flag); atomicAdd(&ctl->full_pairs, (unsigned long long)v_sum); }
         }
