@@ -122,7 +122,10 @@ typedef struct rr_config {
                               runs double -- 1, 2, 4, ... up to force_max_run calls -- with one
                               tested call between two runs; a tested call below the threshold
                               resets the run length; rr_route_anchor clears a pending run.
-                              0 = off.  Not available together with debug_outputs bit 5.      */
+                              0 = off.  Not available together with debug_outputs bit 5.  The
+                              state alternates between two slots from call to call, chosen when the
+                              call is made: a captured sequence of layer calls that is replayed has
+                              to hold an even number of them (without the policy: any number)  */
   int32_t force_max_run;   /* longest forced run (values < 1 count as 1)                       */
 } rr_config;
 

@@ -91,6 +91,9 @@ bool uses_f32(const rr_config* cfg) {
   return !(cfg->debug_outputs & (2 | 4)) && rr_route_f32_supported(shape_params(cfg));
 }
 
+// Words per row tile of the flagged rows' counts: the fp32 kernel's CTAs have 8 or 16 rows and store a byte each.
+int count_words(const rr_config* cfg) { return uses_f32(cfg) ? RR_ROW_TILE / 8 / 4 : 1; }
+
 bool uses_sweep(const rr_config* cfg) {
   return (cfg->debug_outputs & 32) && !(cfg->debug_outputs & (2 | 16)) && rr_route_sweep_supported(shape_params(cfg));
 }
@@ -126,7 +129,7 @@ Layout make_layout(const rr_config* c) {
   L.refresh_rows = o;    o = align_up(o + rows * 4);
   L.refresh_count = o;   o = align_up(o + 4);
   L.problem_offsets = o; o = align_up(o + (P + 1) * 4);
-  L.tile_counts = o;     o = align_up(o + 2 * tiles * 4);
+  L.tile_counts = o;     o = align_up(o + tiles * 4 * count_words(c));
   L.counters = o;        o = align_up(o + RR_NUM_COUNTERS * 8);
   L.status = o;          o = align_up(o + 4);
   L.force_state = o;     o = align_up(o + 8 * 4);
@@ -161,7 +164,6 @@ int route_layer(rr_ledger* L, const void* qc, const void* kc, int layer, bool an
   RRParams p = L->p;
   p.force_in = p.force_stats + 2 * (L->call_index & 1u);
   p.force_out = p.force_stats + 2 * ((L->call_index + 1u) & 1u);
-  if (L->call_index & 1u) { int32_t* t = p.tile_counts; p.tile_counts = p.tile_counts_next; p.tile_counts_next = t; }
   ++L->call_index;
   // LAUNCH(kind, call): enqueue one kernel, bracketed by events while profiling
 #define LAUNCH(kind, call)                                                         \
@@ -316,8 +318,8 @@ int rr_ledger_init(const rr_config* cfg, void* dev_ledger, size_t ledger_bytes,
   p.refresh_rows = (int32_t*)(sb + lay.refresh_rows);
   p.refresh_count = (int32_t*)(sb + lay.refresh_count);
   p.problem_offsets = (int32_t*)(sb + lay.problem_offsets);
-  p.tile_counts = (int32_t*)(sb + lay.tile_counts);
-  p.tile_counts_next = p.tile_counts + p.n_tiles;     // (swapped every other call, route_layer)
+  p.tile_counts = (uint32_t*)(sb + lay.tile_counts);
+  p.count_words = count_words(cfg);
   p.counters = (unsigned long long*)(sb + lay.counters);
   p.status = (uint32_t*)(sb + lay.status);
   p.force_stats = (int32_t*)(sb + lay.force_state);

@@ -26,7 +26,9 @@ struct RRParams {
   // per-layer outputs and scratch
   uint8_t* flags; float* alpha; float* beta; float* tau;
   int32_t* refresh_rows; int32_t* refresh_count; int32_t* problem_offsets;
-  int32_t* tile_counts; int32_t* tile_counts_next;   // flagged rows per row tile of this call / the next one
+  // Flagged rows per row tile of this call: the sum of the bytes of count_words words.  Who counts stores plainly, a word
+  // per tile or a byte per part of one (rr_store_count), so that a call needs nothing of the one before it.
+  uint32_t* tile_counts; int count_words;
   int32_t* token_ranges; float* cand_scores;
   unsigned long long* counters; uint32_t* status;
   float* S;                                // [rows, n_k] score rows of the two-pass path
@@ -72,6 +74,16 @@ __host__ __device__ __forceinline__ int rr_valid_count(int i, int n_k, int causa
   // (an offset beyond n_k gives every row all chunks; 32 bits are enough then)
   const int o = off < n_k ? off : n_k, v = i + 1 + o;
   return !causal || v > n_k ? n_k : v;
+}
+
+// The count of a CTA that owns the rows row0 .. row0 + rows - 1 of a problem, a part of a row tile: n goes to the first of
+// the bytes that stand for these rows (32 of them each, 8 where a tile has four words), 0 to the others and, behind the
+// problem's last row, to the rest of the tile's.
+__device__ __forceinline__ void rr_store_count(const RRParams& p, int prob, int row0, int rows, int n) {
+  const int bytes = 4 * p.count_words, per = RR_ROW_TILE / bytes, first = row0 % RR_ROW_TILE / per;
+  uint8_t* const c = (uint8_t*)(p.tile_counts + (size_t)(prob * p.tiles_per_problem + row0 / RR_ROW_TILE) * p.count_words);
+  const int end = row0 + rows >= p.n_q ? bytes : first + rows / per;
+  for (int b = first; b < end; ++b) c[b] = (uint8_t)(b == first ? n : 0);
 }
 
 // Monotone map float -> uint32 (larger float <=> larger key); -0.0 is folded onto +0.0.

@@ -10,7 +10,7 @@ constexpr unsigned FULL = 0xFFFFFFFFu;
 
 // ---- compaction -----------------------------------------------------------------------
 // One CTA per row tile (RR_ROW_TILE rows of one problem).  The tile's base offset is the sum
-// of the flagged counts of all earlier tiles (written by the rescoring kernel); inside the
+// of the flagged counts of all earlier tiles (written by the kernel that tested the rows); inside the
 // tile a ballot/popcount scan gives each flagged row its slot.  The list is therefore in
 // ascending global row id -- exactly numpy.nonzero(flags) -- with no atomics and no waits
 // (the price: n_tiles^2 / 2 count reads in total, nothing at the few thousand tiles of a layer).
@@ -24,7 +24,6 @@ compact_kernel(RRParams p, unsigned long long dense_pairs) {
   const int prob = tile_id / p.tiles_per_problem, tile = tile_id % p.tiles_per_problem;
   rr_pdl_wait();
   rr_pdl_trigger();
-  if (tid == 0) p.tile_counts_next[tile_id] = 0;       // (for kernels that add to the counts)
 
   // Forced anchor (Section 3.2, policy of rr_config.force_permille): the previous tested relay
   // flagged so many rows that this call routes every row.  The tile does what the anchor's fill
@@ -62,11 +61,18 @@ compact_kernel(RRParams p, unsigned long long dense_pairs) {
   const bool in = i < p.n_q;
   const bool f = in && p.flags[g] != 0;
   const int age = in ? p.ages[g] : 0;
-  int part = 0;
-  for (int t = tid; t < tile_id; t += RR_ROW_TILE) part += p.tile_counts[t];
+  unsigned part = 0;                                         // (bytes: see RRParams)
+  if (p.count_words == 1) {
+    for (int t = tid; t < tile_id; t += RR_ROW_TILE) part = __dp4a(p.tile_counts[t], 0x01010101u, part);
+  } else {
+    for (int t = tid; t < tile_id; t += RR_ROW_TILE) {
+      const uint4 c = reinterpret_cast<const uint4*>(p.tile_counts)[t];
+      part = __dp4a(c.x, 0x01010101u, __dp4a(c.y, 0x01010101u, __dp4a(c.z, 0x01010101u, __dp4a(c.w, 0x01010101u, part))));
+    }
+  }
   part = __reduce_add_sync(FULL, part);
   const unsigned bal = __ballot_sync(FULL, f);
-  if (lane == 0) { s_part[warp] = part; s_cnt[warp] = __popc(bal); }
+  if (lane == 0) { s_part[warp] = (int)part; s_cnt[warp] = __popc(bal); }
   __syncthreads();
   int base = 0, before = 0, total = 0;
 #pragma unroll
@@ -103,7 +109,6 @@ __global__ void anchor_fill_kernel(RRParams p, unsigned long long dense_pairs) {
   const float qnan = __int_as_float(0x7fc00000);
   rr_pdl_wait();
   rr_pdl_trigger();
-  if (g < p.n_tiles) p.tile_counts_next[g] = 0;
   if (g < p.rows) {
     p.flags[g] = 1;
     p.refresh_rows[g] = g;
@@ -248,7 +253,7 @@ __global__ void reset_kernel(RRParams p) {
     p.flags[e] = 0; p.alpha[e] = 0.f; p.beta[e] = 0.f; p.refresh_rows[e] = -1;
   }
   for (size_t e = tid; e <= (size_t)p.P; e += stride) p.problem_offsets[e] = 0;
-  for (size_t e = tid; e < (size_t)p.n_tiles; e += stride) { p.tile_counts[e] = 0; p.tile_counts_next[e] = 0; }
+  for (size_t e = tid; e < (size_t)p.n_tiles * p.count_words; e += stride) p.tile_counts[e] = 0;
   if (p.token_ranges)
     for (size_t e = tid; e < (size_t)p.rows * p.k * 2; e += stride) p.token_ranges[e] = -1;
   if (tid < RR_NUM_COUNTERS) p.counters[tid] = 0;

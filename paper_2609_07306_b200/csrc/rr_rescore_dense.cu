@@ -252,7 +252,7 @@ rescore_dense_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q,
 
   pipe.teardown(p);                                           // includes a __syncthreads()
   if (tid == 0) {
-    p.tile_counts[tile_id] = (int)s_cnt[0];
+    p.tile_counts[tile_id] = (uint32_t)s_cnt[0];
     atomicAdd(&p.counters[RR_CNT_FLAGGED_ROWS], s_cnt[0]);
     atomicAdd(&p.counters[RR_CNT_CAND_PAIRS], s_cnt[1]);
     atomicAdd(&p.counters[RR_CNT_FULL_PAIRS], s_cnt[2]);

@@ -248,7 +248,7 @@ rescore_rows_kernel(RRParams p, const __grid_constant__ CUtensorMap tmap_q, cons
   }
   if (tid == 0) {
     if (ctl->abort_flag) atomicOr(p.status, RR_STATUS_TIMEOUT);
-    p.tile_counts[prob * tiles_m + tm] = (int)ctl->flagged;
+    p.tile_counts[prob * tiles_m + tm] = (uint32_t)ctl->flagged;
     atomicAdd(&p.counters[RR_CNT_FLAGGED_ROWS], (unsigned long long)ctl->flagged);
     atomicAdd(&p.counters[RR_CNT_CAND_PAIRS], (unsigned long long)ctl->cand);
     atomicAdd(&p.counters[RR_CNT_FULL_PAIRS], ctl->full_pairs);

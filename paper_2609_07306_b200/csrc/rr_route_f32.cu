@@ -144,8 +144,7 @@ route_f32_kernel(RRParams p, const float* __restrict__ qc, const float* __restri
   if (!all) {
     __syncthreads();
     if (tid == 0) {
-      // (the compaction kernel of the previous call left the counts at zero)
-      if (s_flagged) atomicAdd(&p.tile_counts[prob * p.tiles_per_problem + row0 / RR_ROW_TILE], (int)s_flagged);
+      rr_store_count(p, prob, row0, R, (int)s_flagged);
       atomicAdd(&p.counters[RR_CNT_FLAGGED_ROWS], (unsigned long long)s_flagged);
       atomicAdd(&p.counters[RR_CNT_CAND_PAIRS], (unsigned long long)s_cand);
       atomicAdd(&p.counters[RR_CNT_FULL_PAIRS], s_full);

@@ -880,8 +880,7 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   }
   if (tid == 0 && ctl->abort_flag) atomicOr(p.status, RR_STATUS_TIMEOUT);
   if (tested && tid == 0) {
-    // (several CTAs may share a tile of the list; the previous call's list kernel left the counts at zero)
-    atomicAdd(&p.tile_counts[prob * p.tiles_per_problem + tm * own / RR_ROW_TILE], (int)ctl->flagged);
+    rr_store_count(p, prob, tm * own, own, (int)ctl->flagged);
     atomicAdd(&p.counters[RR_CNT_FLAGGED_ROWS], (unsigned long long)ctl->flagged);
     atomicAdd(&p.counters[RR_CNT_CAND_PAIRS], (unsigned long long)ctl->cand);
     atomicAdd(&p.counters[RR_CNT_FULL_PAIRS], ctl->full_pairs);

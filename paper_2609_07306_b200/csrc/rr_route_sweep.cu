@@ -885,7 +885,7 @@ route_sweep_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   if (warp == 0) {
     if (lane == 0 && ctl->abort_flag) atomicOr(p.status, RR_STATUS_TIMEOUT);
     if (lane == 0 && inplace) {      // what the compaction kernel and the work counters need
-      p.tile_counts[prob * tiles_m + tm] = (int)ctl->n_flagged;
+      p.tile_counts[prob * tiles_m + tm] = (uint32_t)ctl->n_flagged;
       atomicAdd(&p.counters[RR_CNT_FLAGGED_ROWS], (unsigned long long)ctl->n_flagged);
       atomicAdd(&p.counters[RR_CNT_CAND_PAIRS], (unsigned long long)ctl->n_cand);
       atomicAdd(&p.counters[RR_CNT_FULL_PAIRS], ctl->v_flagged);
