@@ -158,7 +158,9 @@ __device__ __forceinline__ void draw_sentinels(const RRParams& p, uint32_t bits,
     }
     // A row with few free chunks needs many draws (65 chunks, 48 of them excluded, 16 to draw: 150):
     // what is left after 4 r draws is drawn by the warp, 32 at a time, a row after the other.
-    __syncwarp();                                          // (all lanes read the marks that this row's lane has made)
+    // (All lanes read the marks of the row's lane: they are visible before the vote, which waits for every lane.  A
+    // __syncwarp() here made whole passes 1-4 % longer, the fence costs nothing.)
+    __threadfence_block();
     unsigned left = __ballot_sync(FULL, dst < end);
 #pragma unroll 1
     while (left) {
