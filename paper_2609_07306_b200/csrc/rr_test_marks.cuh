@@ -7,6 +7,7 @@
 
 // Marks the valid ids of rows row0 .. row0 + n_rows - 1 (of problem prob; ids: the whole array, w per row): the bit
 // of id goes to plane + row * row_pitch + (id / 32) * WORD_PITCH.  The warp is one of PARTS that share the work.
+// (Ordinary loads: the routing kernel writes the same arrays later on, which rules out the read-only path.)
 // Returns how many ids this lane has marked; `bad`: it has met one that its row may not select.
 template <int PARTS, uint32_t WORD_PITCH>
 __device__ __forceinline__ int rr_mark_rows(const RRParams& p, const int32_t* all_ids, int w, int prob, int row0,
@@ -34,7 +35,7 @@ __device__ __forceinline__ int rr_mark_rows(const RRParams& p, const int32_t* al
       int4 q[U];
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        q[u] = f0 + u * STEP < total ? __ldg(reinterpret_cast<const int4*>(ids) + f0 + u * STEP) : make_int4(-1, -1, -1, -1);
+        q[u] = f0 + u * STEP < total ? reinterpret_cast<const int4*>(ids)[f0 + u * STEP] : make_int4(-1, -1, -1, -1);
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int rr = row_of(f0 + u * STEP), vr = valid_of(rr);
@@ -47,7 +48,7 @@ __device__ __forceinline__ int rr_mark_rows(const RRParams& p, const int32_t* al
     for (int f0 = part * 32 + lane; f0 < total; f0 += U * STEP) {
       int q[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) q[u] = f0 + u * STEP < total ? __ldg(ids + f0 + u * STEP) : -1;
+      for (int u = 0; u < U; ++u) q[u] = f0 + u * STEP < total ? ids[f0 + u * STEP] : -1;
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int rr = row_of(f0 + u * STEP);
