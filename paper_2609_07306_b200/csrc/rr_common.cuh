@@ -78,12 +78,14 @@ __host__ __device__ __forceinline__ int rr_valid_count(int i, int n_k, int causa
 
 // The count of a CTA that owns the rows row0 .. row0 + rows - 1 of a problem, a part of a row tile: n goes to the first of
 // the bytes that stand for these rows (32 of them each, 8 where a tile has four words), 0 to the others and, behind the
-// problem's last row, to the rest of the tile's.
+// problem's last row, to the rest of the tile's.  WORDS: p.count_words of the ledgers that the kernel serves.
+template <int WORDS>
 __device__ __forceinline__ void rr_store_count(const RRParams& p, int prob, int row0, int rows, int n) {
-  const int bytes = 4 * p.count_words, per = RR_ROW_TILE / bytes, first = row0 % RR_ROW_TILE / per;
-  uint8_t* const c = (uint8_t*)(p.tile_counts + (size_t)(prob * p.tiles_per_problem + row0 / RR_ROW_TILE) * p.count_words);
+  constexpr int bytes = 4 * WORDS, per = RR_ROW_TILE / bytes;
+  const int first = row0 % RR_ROW_TILE / per;
+  uint8_t* const c = (uint8_t*)(p.tile_counts + (size_t)(prob * p.tiles_per_problem + row0 / RR_ROW_TILE) * WORDS);
   const int end = row0 + rows >= p.n_q ? bytes : first + rows / per;
-  for (int b = first; b < end; ++b) c[b] = (uint8_t)(b == first ? n : 0);
+  for (int b = first; b < end; ++b) c[b] = (uint8_t)n, n = 0;
 }
 
 // Monotone map float -> uint32 (larger float <=> larger key); -0.0 is folded onto +0.0.

@@ -430,6 +430,10 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   };
   auto acc_addr = [&](int gt) -> uint32_t { return acc_lane + (uint32_t)((gt % ACC_STAGES) * BN + side * SLICE); };
 
+  // The quarter's byte among the flagged counts (stored as soon as it is known: at the kernel's end it was 0.4 us late).
+  uint8_t* const count = (uint8_t*)(p.tile_counts + prob * p.tiles_per_problem) + (tm * own >> 5) + quarter;
+  static_assert(RR_ROW_TILE == 128, "a byte of the tile's word per quarter");
+
   if (warp == 0) {
     // The Kc tiles beyond the ring are asked into L2, and so are the Qc rows of the CTA that will
     // start about when this one ends (CTAs start in index order as SMs fall free: the one that comes
@@ -459,6 +463,9 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
     // A quarter without a row to route (the end of a refresh list, a ragged last tile) only hands its
     // accumulators back.  All of its warps come here, so nobody waits for them at its barriers
     // (3 % of 256 x 256 rows on the list: 24.9 -> 24.1 us).
+    // (rows behind the problem's last one, in the same row tile, are none of another CTA's)
+    if (tested && j == 0 && lane == 0 && tm * own + quarter * 32 >= p.n_q && (tm * own & (RR_ROW_TILE - 1)) + quarter * 32 < RR_ROW_TILE)
+      *count = 0;
 #pragma unroll 1
     for (int first = 0; first < 2 * n_tiles; first += n_tiles)
 #pragma unroll 1
@@ -581,7 +588,7 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
         if (j == 0) {
           if (row >= 0 && stands) { p.flags[g] = routed ? 1 : 0; p.alpha[g] = amin; p.beta[g] = bmax; }
           const int n_flag = __popc(__ballot_sync(FULL, routed)), v_sum = __reduce_add_sync(FULL, routed ? v : 0);
-          if (lane == 0) { atomicAdd(&ctl->flagged, (uint32_t)n_flag); atomicAdd(&ctl->full_pairs, (unsigned long long)v_sum); }
+          if (lane == 0) { *count = (uint8_t)n_flag; atomicAdd(&ctl->flagged, (uint32_t)n_flag); atomicAdd(&ctl->full_pairs, (unsigned long long)v_sum); }
         }
         if (!__any_sync(FULL, routed)) {                     // (the quarter's four warps agree)
 #pragma unroll 1
@@ -880,7 +887,6 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   }
   if (tid == 0 && ctl->abort_flag) atomicOr(p.status, RR_STATUS_TIMEOUT);
   if (tested && tid == 0) {
-    rr_store_count(p, prob, tm * own, own, (int)ctl->flagged);
     atomicAdd(&p.counters[RR_CNT_FLAGGED_ROWS], (unsigned long long)ctl->flagged);
     atomicAdd(&p.counters[RR_CNT_CAND_PAIRS], (unsigned long long)ctl->cand);
     atomicAdd(&p.counters[RR_CNT_FULL_PAIRS], ctl->full_pairs);
