@@ -95,7 +95,9 @@ typedef struct rr_config {
                               time-out and the status word gets RR_STATUS_TIMEOUT;
                               bit 9 (tests): the same for a wait that expires while the first
                               relay whose test runs inside the routing kernel decides about its
-                              rows                                                          */
+                              rows;
+                              bit 10: a relay tests its rows in a kernel of its own, with the list
+                              between it and the routing kernel, on small grids as well        */
   /* Optional policies either side of the trigger; all zero = the plain method.             */
   int32_t global_sentinels;/* mandatory global candidates (Section 3.1, item 3): bit 0 = the
                               sink chunk 0, bit 1 = the most recent chunk the row may select.

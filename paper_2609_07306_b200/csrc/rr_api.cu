@@ -340,7 +340,7 @@ int rr_ledger_init(const rr_config* cfg, void* dev_ledger, size_t ledger_bytes,
   const bool strip = !(cfg->debug_outputs & 4);
   L->rows_rescore = strip && !L->fused && rr_rescore_rows_supported(p);
   L->dense_rescore = strip && L->fused && rr_rescore_dense_supported(p);
-  L->tests = L->rows && L->rows_rescore && rr_route_quad_tests(p);
+  L->tests = L->rows && L->rows_rescore && !(cfg->debug_outputs & 1024) && rr_route_quad_tests(p);
   *out = L;
   return RR_OK;
 }
