@@ -76,12 +76,13 @@ constexpr uint32_t WORD_PITCH = BM * 4;            // [word][row] areas
 __host__ __device__ constexpr int stages_of(int d, int ctas) { return d == 64 || ctas == 1 ? 3 : 2; }   // of the Kc ring
 
 struct Ctl {
-  uint64_t full[MAX_STAGES], acc_full[ACC_STAGES], acc_empty[ACC_STAGES], drain;
+  uint64_t full[MAX_STAGES], acc_full[ACC_STAGES], acc_empty[ACC_STAGES], drain, decided;
   uint32_t tmem_base, abort_flag, hard_n, pad_;
   uint8_t cnt[TPR][BM];                 // survivors per thread; after the cuts [0], [1]: cut k / k + m undecided
   uint8_t hard_rows[BM];                // rows handed to the slow path, in registration order
   int8_t hard_slot[BM];                 // position of a row in hard_rows, -1 = none
   uint8_t gave_up[BM / 32];             // of the test: a warp of the quarter has met a wait that gave up,
+  uint32_t any_routed;                  // a row of the CTA failed,
   uint32_t flagged, cand;               // rows that failed, candidates looked at,
   unsigned long long full_pairs;        // valid chunks of the rows that failed
 };
@@ -255,6 +256,8 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
     ctl->hard_n = 0;
     ctl->flagged = 0; ctl->cand = 0; ctl->full_pairs = 0ull;
     for (int q = 0; q < BM / 32; ++q) ctl->gave_up[q] = 0;
+    ctl->any_routed = 0;
+    mbar_init(&ctl->decided, BM / 32);                     // one arrival per quarter
     mbar_fence_init();
   }
   if ((smem_u32(smem) & 1023u) != 0u) {                    // reported like a wait that gave up
@@ -365,11 +368,19 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   // says: tile gt may be fetched once tile gt - STAGES is complete.  (That barrier cannot run ahead
   // of the wait: its next completion is tile gt - STAGES + ACC_STAGES >= gt, not fetched yet.)
   // Both roles are run by whole, converged warps (see umma_bf16_ts_warp).
+  // Sweep 2 of a CTA that tests its rows begins when its quarters have decided, and does not if all of them pass
+  // (a wait that gives up ends it as well).  Called by whole warps.  What fails is sorted meanwhile, so that nobody
+  // waits (8 x 256 x 256 at 83 % and 15 x 389 x 777 at 55 % failing: no difference).  With no row failing, six layers:
+  // 7 x 1345 x 1915 202 -> 181 us, 1 x 202 x 1362 176 -> 154, 8 x 200 x 256 79 -> 75.
+  auto sweep2 = [&]() -> bool {
+    return __all_sync(FULL, mbar_wait_spin(&ctl->decided, 0, abort_flag)) && *(volatile uint32_t*)&ctl->any_routed != 0u;
+  };
   auto produce = [&](int first, int count, int begin) {
     int t = begin % n_tiles, s = begin % STAGES, gt = begin;
 #pragma unroll 1
     for (; gt < first + count; ++gt) {
       const int done = gt - STAGES;
+      if (tested && done == n_tiles && !sweep2()) break;   // (first tile that needs an MMA of sweep 2)
       if (done >= first &&
           !__all_sync(FULL, mbar_wait_spin(&ctl->acc_full[done % ACC_STAGES], (done / ACC_STAGES) & 1, abort_flag))) break;
       tma_load_tile_warp(ring + s * TILE, tmap_ptr, t * BN, prob, &ctl->full[s], TILE);
@@ -390,6 +401,7 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
 #pragma unroll 1
     for (int gt = first; gt < first + count; ++gt) {
       const int as = gt % ACC_STAGES, s = gt % STAGES;
+      if (tested && gt == n_tiles && !sweep2()) return;
       if (!__all_sync(FULL, mbar_wait_spin(&ctl->acc_empty[as], ((gt / ACC_STAGES) & 1) ^ 1, abort_flag))) return;
       if (!__all_sync(FULL, mbar_wait_spin(&ctl->full[s], (gt / STAGES) & 1, abort_flag))) return;
       tc_fence_after();
@@ -466,10 +478,13 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
     // (rows behind the problem's last one, in the same row tile, are none of another CTA's)
     if (tested && j == 0 && lane == 0 && tm * own + quarter * 32 >= p.n_q && (tm * own & (RR_ROW_TILE - 1)) + quarter * 32 < RR_ROW_TILE)
       *count = 0;
+    if (tested && j == 0 && lane == 0) mbar_arrive(&ctl->decided);
 #pragma unroll 1
-    for (int first = 0; first < 2 * n_tiles; first += n_tiles)
+    for (int first = 0; first < 2 * n_tiles; first += n_tiles) {
+      if (tested && first > 0 && !sweep2()) break;
 #pragma unroll 1
       for (int t = pair; t < n_tiles && tile_wait(first + t); t += 2) tile_release(first + t);
+    }
   } else do {
     PH_T0();
 #ifdef RR_PHASE_TIMING
@@ -585,12 +600,20 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
           bmax = fmaxf(bmax, ldsf(slot(TPR + t) + 4u));
         }
         routed = row >= 0 && stands && rr_challenge(p, g, amin, bmax);
+        const unsigned failed = __ballot_sync(FULL, routed); // (the quarter's four warps agree)
         if (j == 0) {
           if (row >= 0 && stands) { p.flags[g] = routed ? 1 : 0; p.alpha[g] = amin; p.beta[g] = bmax; }
-          const int n_flag = __popc(__ballot_sync(FULL, routed)), v_sum = __reduce_add_sync(FULL, routed ? v : 0);
-          if (lane == 0) { *count = (uint8_t)n_flag; atomicAdd(&ctl->flagged, (uint32_t)n_flag); atomicAdd(&ctl->full_pairs, (unsigned long long)v_sum); }
+          const int n_flag = __popc(failed), v_sum = __reduce_add_sync(FULL, routed ? v : 0);
+          if (lane == 0) {
+            if (failed) ctl->any_routed = 1;
+            mbar_arrive(&ctl->decided);
+            *count = (uint8_t)n_flag;
+            atomicAdd(&ctl->flagged, (uint32_t)n_flag);
+            atomicAdd(&ctl->full_pairs, (unsigned long long)v_sum);
+          }
         }
-        if (!__any_sync(FULL, routed)) {                     // (the quarter's four warps agree)
+        if (failed == 0u) {                                  // sweep 2's accumulators go back, if another quarter needs it
+          if (!sweep2()) break;
 #pragma unroll 1
           for (int t = pair; t < n_tiles && tile_wait(n_tiles + t); t += 2) tile_release(n_tiles + t);
           break;
