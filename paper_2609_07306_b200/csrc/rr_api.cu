@@ -92,7 +92,7 @@ bool uses_f32(const rr_config* cfg) {
 }
 
 // Words per row tile of the flagged rows' counts: the fp32 kernel's CTAs have 8 or 16 rows and store a byte each.
-int count_words(const rr_config* cfg) { return uses_f32(cfg) ? RR_ROW_TILE / 8 / 4 : 1; }
+int count_words(const rr_config* cfg) { return uses_f32(cfg) ? RR_COUNT_WORDS_F32 : 1; }
 
 bool uses_sweep(const rr_config* cfg) {
   return (cfg->debug_outputs & 32) && !(cfg->debug_outputs & (2 | 16)) && rr_route_sweep_supported(shape_params(cfg));

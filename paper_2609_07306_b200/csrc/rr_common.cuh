@@ -9,6 +9,7 @@
 
 #define RR_ROW_TILE 128            // rows per compaction / rescoring tile (per problem)
 #define RR_MAX_NK 4096
+#define RR_COUNT_WORDS_F32 4           // words of a row tile's flagged count in the fp32 kernel: a byte per 8 rows
 #define RR_MAX_C 256
 
 // Everything a kernel needs to know about one ledger; passed by value.

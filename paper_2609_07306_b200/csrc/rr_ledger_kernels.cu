@@ -16,6 +16,7 @@ constexpr unsigned FULL = 0xFFFFFFFFu;
 // (the price: n_tiles^2 / 2 count reads in total, nothing at the few thousand tiles of a layer).
 // The same pass advances the ages (flagged -> 0, stable -> +1) and, once per launch, the
 // per-layer counters: nothing later in the layer reads either.
+template <int WORDS>                                         // p.count_words
 __global__ void __launch_bounds__(RR_ROW_TILE)
 compact_kernel(RRParams p, unsigned long long dense_pairs) {
   __shared__ int s_part[RR_ROW_TILE / 32], s_cnt[RR_ROW_TILE / 32];   // earlier tiles' counts, by warp; this tile's
@@ -59,10 +60,10 @@ compact_kernel(RRParams p, unsigned long long dense_pairs) {
   const int i = tile * RR_ROW_TILE + tid;
   const int g = prob * p.n_q + i;
   const bool in = i < p.n_q;
-  const bool f = in && p.flags[g] != 0;
+  const int flag = in ? p.flags[g] : 0;
   const int age = in ? p.ages[g] : 0;
   unsigned part = 0;                                         // (bytes: see RRParams)
-  if (p.count_words == 1) {
+  if constexpr (WORDS == 1) {
     for (int t = tid; t < tile_id; t += RR_ROW_TILE) part = __dp4a(p.tile_counts[t], 0x01010101u, part);
   } else {
     for (int t = tid; t < tile_id; t += RR_ROW_TILE) {
@@ -71,6 +72,7 @@ compact_kernel(RRParams p, unsigned long long dense_pairs) {
     }
   }
   part = __reduce_add_sync(FULL, part);
+  const bool f = flag != 0;
   const unsigned bal = __ballot_sync(FULL, f);
   if (lane == 0) { s_part[warp] = (int)part; s_cnt[warp] = __popc(bal); }
   __syncthreads();
@@ -264,7 +266,7 @@ __global__ void reset_kernel(RRParams p) {
 }  // namespace
 
 cudaError_t rr_launch_compact(const RRParams& p, unsigned long long dense_pairs, cudaStream_t st) {
-  const cudaError_t e = rr_launch_pdl(compact_kernel, p.n_tiles, RR_ROW_TILE, 0, st, p, dense_pairs);
+  const cudaError_t e = rr_launch_pdl(p.count_words == 1 ? compact_kernel<1> : compact_kernel<RR_COUNT_WORDS_F32>, p.n_tiles, RR_ROW_TILE, 0, st, p, dense_pairs);
   rr_count_launch();
   return e;
 }

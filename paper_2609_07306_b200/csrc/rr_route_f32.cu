@@ -144,7 +144,7 @@ route_f32_kernel(RRParams p, const float* __restrict__ qc, const float* __restri
   if (!all) {
     __syncthreads();
     if (tid == 0) {
-      rr_store_count<RR_ROW_TILE / 8 / 4>(p, prob, row0, R, (int)s_flagged);
+      rr_store_count<RR_COUNT_WORDS_F32>(p, prob, row0, R, (int)s_flagged);
       atomicAdd(&p.counters[RR_CNT_FLAGGED_ROWS], (unsigned long long)s_flagged);
       atomicAdd(&p.counters[RR_CNT_CAND_PAIRS], (unsigned long long)s_cand);
       atomicAdd(&p.counters[RR_CNT_FULL_PAIRS], s_full);
