@@ -363,11 +363,6 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   const uint32_t tmem_base = ctl->tmem_base;
   volatile uint32_t* abort_flag = &ctl->abort_flag;
 
-  // Tiles are numbered through all sweeps (gt): stage and phase of every ring follow from gt.
-  // A stage of the Kc ring is free again when the MMAs of its tile are done, which is what acc_full
-  // says: tile gt may be fetched once tile gt - STAGES is complete.  (That barrier cannot run ahead
-  // of the wait: its next completion is tile gt - STAGES + ACC_STAGES >= gt, not fetched yet.)
-  // Both roles are run by whole, converged warps (see umma_bf16_ts_warp).
   // Sweep 2 of a CTA that tests its rows begins when its quarters have decided, and does not if all of them pass
   // (a wait that gives up ends it as well).  Called by whole warps.  What fails is sorted meanwhile, so that nobody
   // waits (8 x 256 x 256 at 83 % and 15 x 389 x 777 at 55 % failing: no difference).  With no row failing, six layers:
@@ -375,6 +370,11 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   auto sweep2 = [&]() -> bool {
     return __all_sync(FULL, mbar_wait_spin(&ctl->decided, 0, abort_flag)) && *(volatile uint32_t*)&ctl->any_routed != 0u;
   };
+  // Tiles are numbered through all sweeps (gt): stage and phase of every ring follow from gt.
+  // A stage of the Kc ring is free again when the MMAs of its tile are done, which is what acc_full
+  // says: tile gt may be fetched once tile gt - STAGES is complete.  (That barrier cannot run ahead
+  // of the wait: its next completion is tile gt - STAGES + ACC_STAGES >= gt, not fetched yet.)
+  // Both roles are run by whole, converged warps (see umma_bf16_ts_warp).
   auto produce = [&](int first, int count, int begin) {
     int t = begin % n_tiles, s = begin % STAGES, gt = begin;
 #pragma unroll 1
@@ -443,7 +443,7 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
   auto acc_addr = [&](int gt) -> uint32_t { return acc_lane + (uint32_t)((gt % ACC_STAGES) * BN + side * SLICE); };
 
   // The quarter's byte among the flagged counts (stored as soon as it is known: at the kernel's end it was 0.4 us late).
-  uint8_t* const count = (uint8_t*)(p.tile_counts + prob * p.tiles_per_problem) + (tm * own >> 5) + quarter;
+  auto store_count = [&](int n) { ((uint8_t*)(p.tile_counts + prob * p.tiles_per_problem))[(tm * own >> 5) + quarter] = (uint8_t)n; };
   static_assert(RR_ROW_TILE == 128, "a byte of the tile's word per quarter");
 
   if (warp == 0) {
@@ -477,7 +477,7 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
     // (3 % of 256 x 256 rows on the list: 24.9 -> 24.1 us).
     // (rows behind the problem's last one, in the same row tile, are none of another CTA's)
     if (tested && j == 0 && lane == 0 && tm * own + quarter * 32 >= p.n_q && (tm * own & (RR_ROW_TILE - 1)) + quarter * 32 < RR_ROW_TILE)
-      *count = 0;
+      store_count(0);
     if (tested && j == 0 && lane == 0) mbar_arrive(&ctl->decided);
 #pragma unroll 1
     for (int first = 0; first < 2 * n_tiles; first += n_tiles) {
@@ -607,7 +607,7 @@ route_quad_kernel(RRParams p, const __nv_bfloat16* __restrict__ qc,
           if (lane == 0) {
             if (failed) ctl->any_routed = 1;
             mbar_arrive(&ctl->decided);
-            *count = (uint8_t)n_flag;
+            store_count(n_flag);
             atomicAdd(&ctl->flagged, (uint32_t)n_flag);
             atomicAdd(&ctl->full_pairs, (unsigned long long)v_sum);
           }
