@@ -110,6 +110,9 @@ int rr_bucket_set_init(const rr_config* cfg, const int32_t* widths, int32_t n_pr
                         (char*)dev_scratch + B.scratch_offset, B.scratch_bytes, &B.ledger);
   }
   if (rc != RR_OK) { rr_bucket_set_destroy(S); return rc; }
+  long long tiles = 0;                                  // (the buckets run side by side: each is told of the others)
+  for (const auto& B : S->buckets) tiles += B.ledger->p.n_tiles;
+  for (const auto& B : S->buckets) rr_ledger_beside(B.ledger, (int)std::min(tiles - B.ledger->p.n_tiles, 1LL << 30));
   // (without a device there is nothing to overlap: the calls then run in order on the caller's stream)
   bool ok = S->buckets.size() > 1 && cudaEventCreateWithFlags(&S->forked, cudaEventDisableTiming) == cudaSuccess;
   for (size_t b = 1; ok && b < S->buckets.size(); ++b) {

@@ -20,6 +20,7 @@ struct RRParams {
   int dtype, causal, causal_offset, chunk_tokens, debug;   // debug: bit 0 = store candidate scores
   int coalesce;                            // token ranges of adjacent chunks merged
   int rows, tiles_per_problem, n_tiles;    // row tiles of RR_ROW_TILE per problem / in total
+  int side_tiles;                          // row tiles of the ledgers whose calls run beside this one's (buckets)
   float gamma;
   unsigned long long seed;
   // ledger (persistent state, Section 4.1)
@@ -203,6 +204,7 @@ cudaError_t rr_launch_anchor_fill(const RRParams& p, unsigned long long dense_pa
 cudaError_t rr_launch_expand(const RRParams& p, int is_anchor, cudaStream_t st);
 cudaError_t rr_launch_reset(const RRParams& p, cudaStream_t st);
 
+void rr_ledger_beside(rr_ledger* L, int side_tiles);      // this ledger's calls share the SMs with so many other row tiles
 void rr_count_launch(int n = 1);
 
 // SMs of the current device (148 where the query fails).
