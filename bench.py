@@ -175,22 +175,26 @@ class ClockSampler:
 
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the kernels that
 # dominate a high_drift step, from the ncu captures summarised in profiles/
-# (route_rows_high_drift.md, a refresh of 97 % of the rows; rescore_rows_high_drift.md;
-# sentinels_high_drift.md, relay in place only), and the algorithmic bytes per launch of the same
-# launches.  Other workloads report the capture's traffic-to-algorithmic ratio times their own
-# algorithmic bytes and say so.
-NCU_TRAFFIC_BYTES = {"route_fused": (212.0e6, 196.7e6),
-                     "rescore_dense": (238.3e6, 203.7e6),
-                     "sentinels": (66.5e6, 0.971 * 262144 * 64 * 4)}
+# (route_quad.md, a refresh of 97 % of the rows; rescore_rows_high_drift.md;
+# sentinels_high_drift.md, relay in place only), the algorithmic bytes per launch of the same
+# launches, and the kernel captured.  Other workloads that the same kernel serves report the capture's
+# traffic-to-algorithmic ratio times their own algorithmic bytes and say so; no other kernel's
+# launches are given these figures.
+NCU_TRAFFIC_BYTES = {"route_fused": (213.9e6, 196.7e6, "route_quad_kernel"),
+                     "rescore_dense": (238.3e6, 203.7e6, "rescore_rows_kernel"),
+                     "sentinels": (66.5e6, 0.971 * 262144 * 64 * 4, "sentinel kernel")}
 
 
-def _traffic(kind, workload_name, alg_bytes_per_launch, truncated):
+def _traffic(kind, w, args, alg_bytes_per_launch):
     if kind not in NCU_TRAFFIC_BYTES or alg_bytes_per_launch is None:
         return None, None
-    measured, alg = NCU_TRAFFIC_BYTES[kind]
-    if workload_name == "high_drift" and not truncated:
-        return measured, "ncu capture (profiles/)"
-    return measured / alg * alg_bytes_per_launch, "scaled from the high_drift capture by algorithmic bytes"
+    measured, alg, kernel = NCU_TRAFFIC_BYTES[kind]
+    default_path = not (args.streaming or args.inplace or args.two_pass or args.gathered)
+    if kind != "sentinels" and not (default_path and w.dtype == W.DTYPE_BF16 and 29 <= w.k + max(w.m, 1) <= 96):
+        return None, None
+    if w.name == "high_drift" and not args.layers:
+        return measured, "ncu capture of %s (profiles/)" % kernel
+    return measured / alg * alg_bytes_per_launch, "scaled from the high_drift capture of %s by algorithmic bytes" % kernel
 
 
 # ----------------------------------------------------------------------------- roofline
@@ -404,7 +408,7 @@ def run_ours(args) -> None:
             kernels[kind]["hbm_achieved_gbs"] = r["hbm_achieved_gbs"]
             kernels[kind]["hbm_frac"] = r["hbm_frac"]
         kernels[kind]["alg_bytes_per_launch"] = r.get("alg_bytes_per_launch")
-        tr, src = _traffic(kind, w.name, r.get("alg_bytes_per_launch"), bool(args.layers))
+        tr, src = _traffic(kind, w, args, r.get("alg_bytes_per_launch"))
         if tr is not None:
             kernels[kind]["traffic"] = tr
             kernels[kind]["traffic_source"] = src
