@@ -260,11 +260,6 @@ int route_layer(rr_ledger* L, const void* qc, const void* kc, int layer, bool an
 
 }  // namespace
 
-void rr_ledger_beside(rr_ledger* L, int side_tiles) {
-  L->p.side_tiles = side_tiles;
-  L->tests = L->rows && L->rows_rescore && !(L->cfg.debug_outputs & 1024) && rr_route_quad_tests(L->p);
-}
-
 void rr_count_launch(int n) { g_launches.fetch_add((unsigned long long)n); }
 
 std::mutex& rr_attr_mutex() {
@@ -345,7 +340,7 @@ int rr_ledger_init(const rr_config* cfg, void* dev_ledger, size_t ledger_bytes,
   const bool strip = !(cfg->debug_outputs & 4);
   L->rows_rescore = strip && !L->fused && rr_rescore_rows_supported(p);
   L->dense_rescore = strip && L->fused && rr_rescore_dense_supported(p);
-  rr_ledger_beside(L, 0);
+  L->tests = L->rows && L->rows_rescore && !(cfg->debug_outputs & RR_DEBUG_LIST) && rr_route_quad_tests(p);
   *out = L;
   return RR_OK;
 }

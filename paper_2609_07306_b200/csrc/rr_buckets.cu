@@ -39,6 +39,14 @@ struct rr_bucket_set {
 namespace {
 
 constexpr size_t kAlign = 256;
+
+// Where a relay tests its rows: a ledger alone does it inside the routing kernel up to a row tile per SM
+// (rr_route_quad_tests).  The buckets of a set run side by side and count together, up to half of a B200's 148 SMs: they
+// fill each other's latencies with the list between test and routing as well, and inside, three grids of up to a
+// CTA per SM share the SMs.  Three buckets, six layers, inside against list: 36 row tiles in all, 1525 x 745 242 and 302 us;
+// 48, 209 x 1917 370 and 533; 90, 337 x 186 277 and 230; 108, 160 x 2031 562 and 505; 168, 1754 x 1709 602 and 500; 342,
+// 301 x 628 468 and 394.
+constexpr int MOST_TILES_TESTED_INSIDE = 74;
 size_t up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 // Buckets (ascending width) and bucket-major order of the problems.  widths[p] >= 1.
@@ -104,15 +112,15 @@ int rr_bucket_set_init(const rr_config* cfg, const int32_t* widths, int32_t n_pr
         scratch_bytes < last.scratch_offset + up(last.scratch_bytes))
       rc = RR_ERR_TOO_SMALL;
   }
+  const bool list = S->buckets.size() > 1 &&
+                    (long long)n_problems * ((cfg->n_q + RR_ROW_TILE - 1) / RR_ROW_TILE) > MOST_TILES_TESTED_INSIDE;
   for (size_t b = 0; rc == RR_OK && b < S->buckets.size(); ++b) {
     auto& B = S->buckets[b];
+    if (list) B.cfg.debug_outputs |= RR_DEBUG_LIST;
     rc = rr_ledger_init(&B.cfg, (char*)dev_ledger + B.ledger_offset, B.ledger_bytes,
                         (char*)dev_scratch + B.scratch_offset, B.scratch_bytes, &B.ledger);
   }
   if (rc != RR_OK) { rr_bucket_set_destroy(S); return rc; }
-  long long tiles = 0;                                  // (the buckets run side by side: each is told of the others)
-  for (const auto& B : S->buckets) tiles += B.ledger->p.n_tiles;
-  for (const auto& B : S->buckets) rr_ledger_beside(B.ledger, (int)std::min(tiles - B.ledger->p.n_tiles, 1LL << 30));
   // (without a device there is nothing to overlap: the calls then run in order on the caller's stream)
   bool ok = S->buckets.size() > 1 && cudaEventCreateWithFlags(&S->forked, cudaEventDisableTiming) == cudaSuccess;
   for (size_t b = 1; ok && b < S->buckets.size(); ++b) {

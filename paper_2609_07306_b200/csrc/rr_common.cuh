@@ -11,6 +11,7 @@
 #define RR_MAX_NK 4096
 #define RR_COUNT_WORDS_F32 4           // words of a row tile's flagged count in the fp32 kernel: a byte per 8 rows
 #define RR_MAX_C 256
+#define RR_DEBUG_LIST 1024             // debug_outputs: a relay's test in a kernel of its own, with the list behind it
 
 // Everything a kernel needs to know about one ledger; passed by value.
 struct RRParams {
@@ -20,7 +21,6 @@ struct RRParams {
   int dtype, causal, causal_offset, chunk_tokens, debug;   // debug: bit 0 = store candidate scores
   int coalesce;                            // token ranges of adjacent chunks merged
   int rows, tiles_per_problem, n_tiles;    // row tiles of RR_ROW_TILE per problem / in total
-  int side_tiles;                          // row tiles of the ledgers whose calls run beside this one's (buckets)
   float gamma;
   unsigned long long seed;
   // ledger (persistent state, Section 4.1)
@@ -55,8 +55,8 @@ struct rr_ledger {
   bool rows;                               // full routing runs in the kernels with two CTAs per SM: two threads per
   bool quad;                               // row, or four (wider routes)
   bool tests;                              // relay: challenge test inside the routing kernel with four threads per row
-  bool sweep;                              // ... else in the four-threads-per-row kernel
-  bool inplace;                            // relay: challenge test inside the routing kernel
+  bool sweep;                              // ... else in the kernel of the relay in place (rr_route_sweep.cu)
+  bool inplace;                            // relay: challenge test inside that kernel
   bool fused;                              // ... else in the streaming fused kernel
   bool f32;                                // fp32 inputs: test and routing in one kernel
   bool rows_rescore;                       // relay rescoring reads the tensor-core score strip
@@ -204,7 +204,6 @@ cudaError_t rr_launch_anchor_fill(const RRParams& p, unsigned long long dense_pa
 cudaError_t rr_launch_expand(const RRParams& p, int is_anchor, cudaStream_t st);
 cudaError_t rr_launch_reset(const RRParams& p, cudaStream_t st);
 
-void rr_ledger_beside(rr_ledger* L, int side_tiles);      // this ledger's calls share the SMs with so many other row tiles
 void rr_count_launch(int n = 1);
 
 // SMs of the current device (148 where the query fails).

@@ -63,17 +63,14 @@ bool rr_route_quad_supported(const RRParams& p) { Plan pl; return plan(p, pl); }
 // A relay's test inside the routing kernel: every row goes through sweep 1 there, and the test, the list and the launch
 // of the routing kernel no longer wait for one another.  Taken where every CTA has an SM to itself, so that the
 // rows that pass keep nobody from working: 8 x 256 x 256, twelve layers 371 -> 260 us (without it 361), 15 x 389 x 777
-// 485 -> 404 (440).  With two CTAs to an SM the list is better, dense or not: 32 x 1024 x 1024, 97 % flagged 1000 us
-// against 1090, 17 % flagged 820 against 1005.  Ledgers whose calls run side by side (buckets) count together, and up to half
-// of the SMs: they fill each other's latencies with the list as well, and three grids of up to a CTA per SM share the
-// SMs here.  Three buckets, six layers, inside against list: 36 tiles in all, 1525 x 745 242 and 302 us; 48, 209 x 1917 370
-// and 533; 90, 337 x 186 277 and 230; 108, 160 x 2031 562 and 505; 168, 1754 x 1709 602 and 500; 342, 301 x 628 468 and
-// 394.  The candidates' bitmaps have to fit the column.
+// 485 -> 404 (440).  (A relay without any failing row is the exception: sweep 1 keeps and sorts its maxima for nothing,
+// 7 x 1345 x 1915, six layers 181 us where the list has 139.)  With two CTAs to an SM the list is better, dense or not:
+// 32 x 1024 x 1024, 97 % flagged 1000 us against 1090, 17 % flagged 820 against 1005.  (Buckets that run side by side
+// have a line of their own, rr_buckets.cu.)  The candidates' bitmaps have to fit the column.
 bool rr_route_quad_tests(const RRParams& p) {
   Plan pl;
   if (!plan(p, pl) || (p.n_k + 31) / 32 > std::max(CAPS[pl.variant], LIST_SLOTS)) return false;
-  const long long tiles = (long long)p.n_tiles + p.side_tiles;
-  return tiles <= (p.side_tiles > 0 ? rr_sm_count() / 2 : rr_sm_count());
+  return p.n_tiles <= rr_sm_count();
 }
 
 cudaError_t rr_launch_route_quad(const RRParams& p, const void* qc, const void* kc, const int32_t* row_list, bool test,
