@@ -90,8 +90,9 @@ typedef struct rr_config {
                               score GEMM over a compacted list); the results are the same;
                               bit 8: accepted, without effect;
                               bits 6, 7 (tests): the first wait of the first CTA of the first
-                              routing launch (bit 6) / strip rescoring launch (bit 7) of this
-                              ledger counts as expired, once: that CTA gives up as after a real
+                              routing launch (bit 6) / launch that tests a relay's rows (bit 7: the
+                              strip rescoring kernel, or the routing kernel with the test inside) of
+                              this ledger counts as expired, once: that CTA gives up as after a real
                               time-out and the status word gets RR_STATUS_TIMEOUT;
                               bit 9 (tests): the same for a wait that expires while the first
                               relay whose test runs inside the routing kernel decides about its

@@ -1,5 +1,5 @@
 // Candidate rescoring + challenge test (Section 3.2, Eq. 5) on the score strip of the tensor cores:
-// the default for bf16.
+// the default for bf16 beyond one row tile per SM (smaller grids test inside the routing kernel, rr_route_quad.cuh).
 //
 // One CTA owns 128 query rows of one problem and walks the key chunks in tiles of 64: warp 0 loads Kc
 // (TMA), warp 1 multiplies (tcgen05.mma, the Qc tile as the A operand in TMEM), warps 2-9 consume.

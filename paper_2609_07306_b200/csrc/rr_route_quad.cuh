@@ -4,7 +4,7 @@
 // challenge test (Eq. 5) on the scores of the first sweep.  The score matrix never leaves the SM.
 //
 // One CTA owns 128 query rows of one problem (consecutive rows, or a segment of the compacted refresh list,
-// Section 4.2) and walks the key chunks in tiles of 64, stopping at the last chunk any of its rows may select.
+// Section 4.2; with TEST on a small grid 32 or 64 consecutive rows, rows_per_test_cta in rr_route_quad.cu) and walks the key chunks in tiles of 64, stopping at the last chunk any of its rows may select.
 //   warp 0     : TMA producer (Kc tiles, 128-byte swizzle, one copy per tile)
 //   warp 1     : issues tcgen05.mma (M=128, N=64, K=16) into a ring of 3 TMEM accumulators; the Qc tile is the
 //                MMA's A operand in TMEM
@@ -34,7 +34,8 @@
 //
 // 256 x 1024 x 1024, keep 48: 277 us (two threads) -> 261; 64 x 2048 x 2048, keep 96: 408 -> 300; the list of 17 % of
 // 256 x 1024 rows: 130 -> 96; 32 x 1024 x 1024 55 -> 50.
-// TEST, 8 x 256 x 256 (16 CTAs, twelve layers): 371 us with the test and the list before the routing kernel, 260 in it.
+// TEST, 8 x 256 x 256 (twelve layers): 371 us with the test and the list before the routing kernel, 260 in it with
+// 128 rows per CTA, 251 with 32.
 //
 // Tried and taken back: 64 rows per CTA with every query row twice in the MMA, two threads per row, four CTAs per
 // SM (high drift 5625 -> 6753 us per 16 layers: every Kc tile comes twice and waits longer); a pair's share of

@@ -1,6 +1,6 @@
 // The RELAY IN PLACE (on request): full routing with the challenge test of Eq. 5 inside the kernel.
-// Anchors and compacted refreshes run rr_route_rows.cu, which covers the same method with two threads
-// per row and two CTAs per SM; this kernel's four threads per row leave one CTA per SM, but between
+// Anchors and compacted refreshes run rr_route_rows.cu or rr_route_quad.cuh, which cover the same method with two
+// or four threads per row and two CTAs per SM; this kernel's four threads per row leave one CTA per SM, but between
 // its sweeps a row's scores of the first sweep can be looked up, which the test in place needs.
 //
 // Full routing of a set of rows in ONE kernel, two sweeps over the key chunks: score GEMM on

@@ -1,6 +1,6 @@
 // Mandatory global sentinels and the seeded random sentinel sample (Section 3.1 items 2 and 3,
 // Section 3.4) of rows whose route and near-miss sentinels have just been written by the
-// four-threads-per-row kernel (rr_route_sweep.cu; the other routing kernels draw themselves).  One
+// kernel of the relay in place (rr_route_sweep.cu; the other routing kernels draw themselves).  One
 // thread per row, in small blocks so that a layer's rows fill every SM with as many warps as its
 // registers allow: a row's draws are accepted strictly in draw
 // order, a serial chain per row that only many rows in flight can hide (inside the routing
